@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(kThreads) blend_fwd_kernel(
         }
         __syncthreads();
         const int cnt = min(kBatch, n - b0);
-        const int nw = warp_list(s_m, cnt, list);
+        const int nw = warp_list<1>(s_m, cnt, list);
         for (int q0 = 0; q0 < nw; q0 += kExitEvery) {
             if (__all_sync(0xffffffffu, done0 && done1)) break;
             const int q1 = min(q0 + kExitEvery, nw);

@@ -81,15 +81,80 @@ __device__ __forceinline__ Rec load_rec(const float4* __restrict__ rec, uint32_t
     return o;
 }
 
-// Warp-local list of the batch entries (in order) whose block mask has this warp's bit.
-__device__ __forceinline__ int warp_list(const uint8_t* s_m, int cnt, uint8_t* list) {
+// ---------------------------------------------------------------------------------------
+// Two pixels at a time: the thread's two vertically adjacent pixels share one register pair and
+// Blackwell's packed FP32 operations (one instruction, each half rounded as the scalar one).
+// ---------------------------------------------------------------------------------------
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float lo2(f32x2 v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi2(f32x2 v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ float rcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// A record as the walks read it (16-byte broadcast loads): the conic scaled and negated so that
+// the walk forms q = -power2 = -log2(e) power >= 0 (negation commutes with rounding: the bits of
+// power2), and the skip bound alpha >= 1/255 <=> q <= qskip.
+struct __align__(16) StagedRec {
+    float4 A;    // u, v, a2 = 0.5 a log2e, b2 = b log2e
+    float4 B;    // c2 = 0.5 c log2e, opacity, r, g
+    float4 C;    // b (blue), qskip
+};
+
+// Writes record g in that form, with its warp_blocks() mask in the low four bits of the result;
+// bit 4: alpha can reach its clamp (o G up to 0.99) or a colour is not finite.
+__device__ __forceinline__ uint32_t stage_rec(const float4* __restrict__ rec, uint32_t g, float tx0,
+                                              float ty0, StagedRec& o) {
+    const float4 r0 = rec[3 * (size_t)g], r1 = rec[3 * (size_t)g + 1], r2 = rec[3 * (size_t)g + 2];
+    o.A = make_float4(r0.x, r0.y, 0.5f * kLog2e * r0.z, kLog2e * r0.w);
+    o.B = make_float4(0.5f * kLog2e * r1.x, r1.y, r1.z, r1.w);
+    // + 0: never the bits of -0
+    *reinterpret_cast<float2*>(&o.C) = make_float2(r2.x, -(r2.w * kLog2e) + 0.0f);
+    const bool careful = !(r1.y < 0.9899f) || !isfinite(r1.z) || !isfinite(r1.w) || !isfinite(r2.x);
+    return warp_blocks(r0, r1, r2.w, tx0, ty0) | (careful ? 16u : 0u);
+}
+
+// power <= 0 and alpha >= 1/255 in one comparison: as unsigned bits, the floats in [0, qskip]
+// are those at most qskip's (negative q and NaN compare above every float; a record with
+// qskip < 0 reaches no block and is never tested).
+__device__ __forceinline__ bool passes(float q, float qskip) {
+    return __float_as_uint(q) <= __float_as_uint(qskip);
+}
+
+// Warp-local list of the batch entries (in order) whose block mask has this warp's bit, entry e
+// stored as e kScale.
+template <int kScale, class T>
+__device__ __forceinline__ int warp_list(const uint8_t* s_m, int cnt, T* list) {
     const unsigned lane = lane_id(), w = threadIdx.x >> 5;
     int nw = 0;
     for (int base = 0; base < cnt; base += 32) {
         const int e = base + (int)lane;
         const bool hit = e < cnt && ((s_m[e] >> w) & 1u);
         const uint32_t bal = __ballot_sync(0xffffffffu, hit);
-        if (hit) list[nw + __popc(bal & lanemask_lt())] = (uint8_t)e;
+        if (hit) list[nw + __popc(bal & lanemask_lt())] = (T)(e * kScale);
         nw += __popc(bal);
     }
     __syncwarp();
