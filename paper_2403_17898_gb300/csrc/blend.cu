@@ -10,10 +10,21 @@
 // skips the Gaussian (or saturates on it) adds a zero weight and keeps its transmittance, which
 // leaves its sums bit-for-bit as a skipped update would.  Lanes of a warp therefore never
 // diverge inside the walk.  A warp stops walking once all its pixels have saturated (checked
-// every 128 records) and the CTA stops loading batches once all of its pixels have.  The
-// kernel is bound by instruction issue (FP32 + MUFU), not by memory.  The optional n_eval
+// every 128 records) and the CTA stops loading batches once all of its pixels have.
+//
+// The kernel is bound by instruction issue (FP32, comparisons and selections), not by memory:
+// about 50 instructions a visit of a warp to an entry, 83 % of the issue slots.  The skip test is
+// one unsigned comparison on the negated exponent, saturation is the sign of T instead of a
+// flag per pixel, and the 0.99 clamp is compiled in only for batches with an opacity that can
+// reach it.  1080p, 2.1M list entries, with n_last: 230 -> 200 us; the 2M-anchor city frame's
+// blend 165 -> 146 us.  (Packed FP32 pairs for T and the weights cost latency on the one chain
+// that is serial, 208 us; list bytes read four at a time cost their unpacking, 233 us.)  Four
+// entries are evaluated at a time for small images, whose few warps wait on latency.
+// The optional n_eval
 // output counts, per pixel, the (pixel, Gaussian) tests the kernel made while the pixel still
 // needed them: the entries of its warp block's list up to the one it saturated on.
+#include <type_traits>
+
 #include "blend_common.cuh"
 
 namespace ogs {
@@ -22,30 +33,88 @@ namespace {
 using namespace blend;
 
 constexpr int kExitEvery = 128;  // records walked between two warp-wide saturation checks
+constexpr int kWalk = 4;         // entries evaluated at a time
+static_assert(kBatch <= 256, "entries are listed as bytes");
 
-// One pixel's compositing step with Gaussian `idx - 1` of the list, branch-free.  Returns the
-// weight alpha T added to the pixel (0 when it skipped the Gaussian or saturated on it).
-template <bool kEval, bool kLast>
-__device__ __forceinline__ float composite(float p2, float o, float cr, float cg, float cb,
-                                           float pskip2, int idx, bool& done, float& T,
-                                           float& C0, float& C1, float& C2, int& last,
-                                           int& tests) {
-    if (kEval) tests += done ? 0 : 1;               // a test this pixel still needed
-    // skip if power > 0 or alpha < 1/255 (power2 < pskip2)
-    const bool pass = !done && p2 <= 0.f && p2 >= pskip2;
-    const float alpha = fminf(0.99f, raw_alpha(o, p2));
-    const float w = alpha * T;
-    const float Tn = T - w;                         // T (1 - alpha)
-    const bool sat = pass && Tn < 1e-4f;            // this Gaussian would saturate the pixel
-    const bool apply = pass && !sat;
-    const float wgt = apply ? w : 0.0f;
-    C0 = fmaf(cr, wgt, C0);
-    C1 = fmaf(cg, wgt, C1);
-    C2 = fmaf(cb, wgt, C2);
-    T = apply ? Tn : T;
-    if (kLast) last = apply ? idx : last;
-    done = done || sat;
-    return wgt;
+// A thread's two vertically adjacent pixels.  T is the transmittance, negative once the pixel
+// has saturated (or lies outside the image): T (1 - alpha) then falls below every bound by
+// itself, so the walk needs no flag beside it.
+struct Pixels {
+    float fx, fy;                       // the upper one's coordinates
+    float T[2], C[2][3];
+    int last[2], tests[2];
+    __device__ __forceinline__ bool done() const { return T[0] < 0.f && T[1] < 0.f; }
+};
+
+// One compositing step of both pixels with the list's entry number idx - 1, branch-free.
+// wgt receives the weights alpha T added (0 where the pixel skipped the Gaussian or saturated on
+// it).  kClamp: the entry's alpha can exceed 0.99.  Only T is carried from entry to entry:
+// two products, a comparison and a selection.
+template <bool kEval, bool kLast, bool kClamp>
+__device__ __forceinline__ void composite(Pixels& p, const float (&q)[2], const float4& B,
+                                          const float2& C, int idx, float (&wgt)[2]) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        if (kEval) p.tests[i] += p.T[i] < 0.f ? 0 : 1;          // a test this pixel still needed
+        const bool pass = passes(q[i], C.y);                    // power <= 0 and alpha >= 1/255
+        float alpha = __fmul_rn(B.y, ex2(-q[i]));
+        if (kClamp) alpha = fminf(0.99f, alpha);
+        const float w = __fmul_rn(alpha, p.T[i]);
+        const float Tn = __fsub_rn(p.T[i], w);                  // T (1 - alpha)
+        const bool apply = pass && Tn >= 1e-4f;                 // else it would saturate the pixel
+        const float stay = pass ? -fabsf(p.T[i]) : p.T[i];
+        wgt[i] = apply ? w : 0.0f;
+        p.T[i] = apply ? Tn : stay;
+        if (kLast) p.last[i] = apply ? idx : p.last[i];
+        p.C[i][0] = fmaf(B.z, wgt[i], p.C[i][0]);
+        p.C[i][1] = fmaf(B.w, wgt[i], p.C[i][1]);
+        p.C[i][2] = fmaf(C.x, wgt[i], p.C[i][2]);
+    }
+}
+
+// Walks the warp's list of nw staged entries front to back, kWalk of them evaluated at a time
+// (independent up to the transmittance chain).
+template <bool kMaxC, bool kEval, bool kLast, bool kClamp>
+__device__ __forceinline__ void walk_list(Pixels& p, const StagedRec* s_rec, const uint8_t* list,
+                                          int nw, int b0, const uint32_t* s_anchor,
+                                          uint32_t* __restrict__ maxc) {
+    auto step = [&](int i, auto n_) {
+        constexpr int kN = decltype(n_)::value;
+        float q[kN][2];
+        float4 B[kN];
+        float2 C[kN];
+        int j[kN];
+#pragma unroll
+        for (int u = 0; u < kN; ++u) {
+            j[u] = list[i + u];
+            const StagedRec& r = s_rec[j[u]];
+            const float4 A = r.A;
+            B[u] = r.B;
+            C[u] = *reinterpret_cast<const float2*>(&r.C);
+            const float dx = A.x - p.fx, dy = A.y - p.fy, ax = __fmul_rn(A.z, dx);
+            q[u][0] = power2(ax, dx, dy, A.w, B[u].x);
+            q[u][1] = power2(ax, dx, dy - 1.0f, A.w, B[u].x);
+        }
+#pragma unroll
+        for (int u = 0; u < kN; ++u) {
+            float wgt[2];
+            composite<kEval, kLast, kClamp>(p, q[u], B[u], C[u], b0 + j[u] + 1, wgt);
+            if (kMaxC) {
+                // contributions are >= 0, so their float bits order like unsigned ints
+                const uint32_t m = __reduce_max_sync(0xffffffffu,
+                                                     __float_as_uint(fmaxf(wgt[0], wgt[1])));
+                if (lane_id() == 0 && m) atomicMax(&maxc[s_anchor[j[u]]], m);
+            }
+        }
+    };
+    for (int q0 = 0; q0 < nw; q0 += kExitEvery) {
+        if (__all_sync(0xffffffffu, p.done())) break;
+        const int q1 = min(q0 + kExitEvery, nw);
+        int i = q0;
+        for (; i + kWalk <= q1; i += kWalk)
+            step(i, std::integral_constant<int, kWalk>());
+        for (; i < q1; ++i) step(i, std::integral_constant<int, 1>());
+    }
 }
 
 template <bool kMaxC, bool kEval, bool kLast>
@@ -57,9 +126,7 @@ __global__ void __launch_bounds__(kThreads) blend_fwd_kernel(
     uint32_t* __restrict__ maxc) {
     pdl_wait();
     pdl_trigger();
-    __shared__ float4 s_a[kBatch];
-    __shared__ float4 s_b[kBatch];
-    __shared__ float2 s_c[kBatch];
+    __shared__ StagedRec s_rec[kBatch];
     __shared__ uint8_t s_m[kBatch];
     __shared__ uint8_t s_list[kThreads / 32][kBatch];
     __shared__ uint32_t s_anchor[kMaxC ? kBatch : 1];
@@ -70,72 +137,45 @@ __global__ void __launch_bounds__(kThreads) blend_fwd_kernel(
     const int px = tx0 + lx;
     const int py = ty0 + ly;
     const bool in0 = px < W && py < H, in1 = px < W && py + 1 < H;
-    const float fx = (float)px, fy = (float)py;
     const uint2 range = tile_range[tile];
     const int n = (int)(range.y - range.x);
     uint8_t* list = s_list[threadIdx.x >> 5];
-    float T0 = 1.f, T1 = 1.f, C00 = 0.f, C01 = 0.f, C02 = 0.f, C10 = 0.f, C11 = 0.f, C12 = 0.f;
-    int last0 = 0, last1 = 0, tests0 = 0, tests1 = 0;
-    bool done0 = !in0, done1 = !in1;
+    Pixels p{(float)px, (float)py, {in0 ? 1.f : -1.f, in1 ? 1.f : -1.f},
+             {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}}, {0, 0}, {0, 0}};
     for (int b0 = 0; b0 < n; b0 += kBatch) {
-        if (__syncthreads_count(done0 && done1) == kThreads) break;
+        if (__syncthreads_and(p.done())) break;
+        bool clamp = false;
         for (int e = threadIdx.x; e < kBatch && b0 + e < n; e += kThreads) {
             const uint32_t g = pair_gauss[range.x + b0 + e];
-            const Rec r = load_rec(rec, g, (float)tx0, (float)ty0);
-            s_a[e] = r.A;
-            s_b[e] = r.B;
-            s_c[e] = r.C;
-            s_m[e] = (uint8_t)r.blocks;
+            const uint32_t m = stage_rec(rec, g, (float)tx0, (float)ty0, s_rec[e]);
+            s_m[e] = (uint8_t)m;
+            clamp = clamp || (m & 16u);
             if (kMaxC) s_anchor[e] = sel_idx[g / (uint32_t)k];
         }
-        __syncthreads();
-        const int cnt = min(kBatch, n - b0);
-        const int nw = warp_list<1>(s_m, cnt, list);
-        for (int q0 = 0; q0 < nw; q0 += kExitEvery) {
-            if (__all_sync(0xffffffffu, done0 && done1)) break;
-            const int q1 = min(q0 + kExitEvery, nw);
-            for (int q = q0; q < q1; ++q) {
-                const int j = list[q];
-                const float4 A = s_a[j];
-                const float4 B = s_b[j];
-                const float2 Cc = s_c[j];
-                const float dx = A.x - fx;
-                const float dy0 = A.y - fy, dy1 = dy0 - 1.0f;
-                const float ax = __fmul_rn(A.z, dx);
-                const float p0 = power2(ax, dx, dy0, A.w, B.x);
-                const float p1 = power2(ax, dx, dy1, A.w, B.x);
-                const int idx = b0 + j + 1;
-                const float c0 = composite<kEval, kLast>(p0, B.y, B.z, B.w, Cc.x, Cc.y, idx, done0, T0,
-                                                  C00, C01, C02, last0, tests0);
-                const float c1 = composite<kEval, kLast>(p1, B.y, B.z, B.w, Cc.x, Cc.y, idx, done1, T1,
-                                                  C10, C11, C12, last1, tests1);
-                if (kMaxC) {
-                    // contributions are >= 0, so their float bits order like unsigned ints
-                    const uint32_t m = __reduce_max_sync(0xffffffffu,
-                                                         __float_as_uint(fmaxf(c0, c1)));
-                    if (lane_id() == 0 && m) atomicMax(&maxc[s_anchor[j]], m);
-                }
-            }
-        }
+        clamp = __syncthreads_or(clamp);
+        const int nw = warp_list<1>(s_m, min(kBatch, n - b0), list);
+        if (clamp) walk_list<kMaxC, kEval, kLast, true>(p, s_rec, list, nw, b0, s_anchor, maxc);
+        else walk_list<kMaxC, kEval, kLast, false>(p, s_rec, list, nw, b0, s_anchor, maxc);
     }
+    const float T0 = fabsf(p.T[0]), T1 = fabsf(p.T[1]);
     const size_t plane = (size_t)W * H;
     if (in0) {
         const size_t pix = (size_t)py * W + px;
-        img[pix] = C00 + T0 * bg0;
-        img[plane + pix] = C01 + T0 * bg1;
-        img[2 * plane + pix] = C02 + T0 * bg2;
+        img[pix] = p.C[0][0] + T0 * bg0;
+        img[plane + pix] = p.C[0][1] + T0 * bg1;
+        img[2 * plane + pix] = p.C[0][2] + T0 * bg2;
         T_final[pix] = T0;
-        if (kLast) n_last[pix] = (uint32_t)last0;
-        if (kEval) n_eval[pix] = (uint32_t)tests0;
+        if (kLast) n_last[pix] = (uint32_t)p.last[0];
+        if (kEval) n_eval[pix] = (uint32_t)p.tests[0];
     }
     if (in1) {
         const size_t pix = (size_t)(py + 1) * W + px;
-        img[pix] = C10 + T1 * bg0;
-        img[plane + pix] = C11 + T1 * bg1;
-        img[2 * plane + pix] = C12 + T1 * bg2;
+        img[pix] = p.C[1][0] + T1 * bg0;
+        img[plane + pix] = p.C[1][1] + T1 * bg1;
+        img[2 * plane + pix] = p.C[1][2] + T1 * bg2;
         T_final[pix] = T1;
-        if (kLast) n_last[pix] = (uint32_t)last1;
-        if (kEval) n_eval[pix] = (uint32_t)tests1;
+        if (kLast) n_last[pix] = (uint32_t)p.last[1];
+        if (kEval) n_eval[pix] = (uint32_t)p.tests[1];
     }
 }
 

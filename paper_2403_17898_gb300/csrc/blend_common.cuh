@@ -31,9 +31,6 @@ __device__ __forceinline__ float ex2(float x) {
     return y;
 }
 
-// raw opacity o G and the clamped alpha
-__device__ __forceinline__ float raw_alpha(float o, float p2) { return __fmul_rn(o, ex2(p2)); }
-
 // Which 8x8 warp blocks of the tile at (tx0, ty0) can hold a pixel with alpha >= 1/255: those
 // met by the bounding box of the ellipse d^T Q d <= 2 ln(255 o), Q = [[a, b], [b, c]] the conic
 // of record r0/r1/r2 (half extents sqrt(2 ln(255 o) (Q^-1)_xx) and sqrt(... (Q^-1)_yy)).  The
@@ -58,27 +55,6 @@ __device__ __forceinline__ uint32_t warp_blocks(const float4& r0, const float4& 
             m |= 1u << w;
     }
     return m;
-}
-
-// A record in the form the inner loop wants: the conic pre-scaled so that
-// power2 = log2(e) * power = dx (a2 dx + b2 dy) + c2 dy^2 and G = ex2(power2), and the skip
-// bound alpha < 1/255 <=> power2 < pskip2.
-struct Rec {
-    float4 A;   // u, v, a2 = -0.5 a log2e, b2 = -b log2e
-    float4 B;   // c2 = -0.5 c log2e, opacity, r, g
-    float2 C;   // b (blue), pskip2 = p_skip log2e
-    uint32_t blocks;   // warp_blocks() of the record for the tile being blended
-};
-
-__device__ __forceinline__ Rec load_rec(const float4* __restrict__ rec, uint32_t g, float tx0,
-                                        float ty0) {
-    const float4 r0 = rec[3 * (size_t)g], r1 = rec[3 * (size_t)g + 1], r2 = rec[3 * (size_t)g + 2];
-    Rec o;
-    o.A = make_float4(r0.x, r0.y, -0.5f * kLog2e * r0.z, -kLog2e * r0.w);
-    o.B = make_float4(-0.5f * kLog2e * r1.x, r1.y, r1.z, r1.w);
-    o.C = make_float2(r2.x, r2.w * kLog2e);
-    o.blocks = warp_blocks(r0, r1, r2.w, tx0, ty0);
-    return o;
 }
 
 // ---------------------------------------------------------------------------------------

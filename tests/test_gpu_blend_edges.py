@@ -1,6 +1,6 @@
-"""Blend backward at the edges of its walk: lists around the staged batch (128 records) and the
-parked group (8 entries), ragged images, clamped opacities, and image gradients that are not
-finite.  Checked against the FP64 oracle."""
+"""Blending at the edges of its walks: lists around the staged batches (256 records forward, 128
+backward), the entries evaluated at a time (4 and 2) and the parked group (8), ragged images,
+clamped opacities, and image gradients that are not finite.  Checked against the FP64 oracle."""
 import numpy as np
 import pytest
 
@@ -51,10 +51,10 @@ def _setup(torch, W, H, G, opac, seed, sigma=(0.8, 10.0)):
 
 # opacities up to 1 reach the 0.99 clamp (zero derivative); up to 0.95 they do not
 @pytest.mark.parametrize("opac", [(0.05, 0.95), (0.9, 1.0)])
-@pytest.mark.parametrize("G", [1, 2, 7, 8, 9, 127, 128, 129, 300])
+@pytest.mark.parametrize("G", [1, 2, 3, 4, 5, 7, 8, 9, 127, 128, 129, 255, 257, 300])
 @pytest.mark.parametrize("W,H", [(33, 17), (16, 16)])
-def test_blend_bwd_list_and_group_edges(torch, W, H, G, opac):
-    r, _, lst, start, uv, bg, _, bwd = _setup(torch, W, H, G, opac, 11 + G)
+def test_blend_list_and_group_edges(torch, W, H, G, opac):
+    r, _, lst, start, uv, bg, t, bwd = _setup(torch, W, H, G, opac, 11 + G)
     fr = oracle.blend(W, H, start, lst, uv, r["conic"], r["opac"], r["colors"], bg)
     dimg = np.random.default_rng(5).normal(size=(3, H, W)).astype(np.float32)
     # FP32 and FP64 may decide differently at a threshold; such pixels take no part.  The clamp
@@ -66,6 +66,10 @@ def test_blend_bwd_list_and_group_edges(torch, W, H, G, opac):
         a, b, c = r["conic"][g].astype(np.float64)
         raw = r["opac"][g] * np.exp(-0.5 * (a * dx * dx + c * dy * dy) - b * dx * dy)
         near |= np.abs(raw - 0.99) < 1e-4
+    ok = ~near
+    assert np.abs(t["img"].cpu().numpy() - fr["img"])[:, ok].max(initial=0) <= 1e-4
+    assert np.abs(t["T"].cpu().numpy() - fr["T"])[ok].max(initial=0) <= 1e-5
+    assert np.array_equal(t["nl"].cpu().numpy()[ok], fr["last"][ok])
     dimg[:, near] = 0
     d = bwd(dimg)
     ref = oracle.blend_bwd(W, H, start, lst, uv, r["conic"], r["opac"], r["colors"], bg, dimg)
