@@ -27,7 +27,9 @@ constexpr int kOffW2 = kOffB1 + kNB1;
 constexpr int kOffB2 = kOffW2 + kNW2;
 
 // per-anchor rows handed from the row pass to the weight pass (f32, 16-byte aligned rows)
-constexpr int kRowY = 112;    // dL/dy of the 110 stacked outputs (+2 zero)
+constexpr int kRowY = 116;    // dL/dy: opacity 0..9, colour 12..41, covariance 44..113 (padding
+                              // between them unused)
+constexpr int kRowCol = 12, kRowCov = 44;
 constexpr int kRowH = 96;     // hidden activations of the three decoders
 constexpr int kRowP = 96;     // dL/d(pre-activation) of the three decoders
 constexpr int kRowZ = 40;     // decoder input z (36, +4 zero)
@@ -62,46 +64,88 @@ __device__ __forceinline__ float sigm(float x) { return 1.0f / (1.0f + __expf(-x
 // out rows of decoder m (opacity 0, colour 1, covariance 2) inside the 110 stacked outputs
 __device__ __forceinline__ int out_base(int m) { return m == 0 ? 0 : (m == 1 ? kK : 4 * kK); }
 __device__ __forceinline__ int dec_of(int row) { return row < kK ? 0 : (row < 4 * kK ? 1 : 2); }
+// stacked output n's place in a dy row, and back (-1: padding)
+__device__ __forceinline__ int out_row(int n) {
+    return n < kK ? n : (n < 4 * kK ? n - kK + kRowCol : n - 4 * kK + kRowCov);
+}
+__device__ __forceinline__ int row_out(int e) {
+    if (e < kRowCol) return e < kK ? e : -1;
+    if (e < kRowCov) return e - kRowCol < 3 * kK ? e - kRowCol + kK : -1;
+    return e - kRowCov < 7 * kK ? e - kRowCov + 4 * kK : -1;
+}
 
-// Gradient of the loss w.r.t. the outputs y of decoder m for Gaussian i of anchor j (row
-// g = r k + i of the Gaussian arrays): opacity w tanh (zero where the opacity was dropped),
-// colour sigmoid, scale l_v sigmoid, unit quaternion; the scale and position terms of l_v and
-// the offsets are accumulated here (dlv, doffs).
+// Gradients of one Gaussian that the decoders' backward starts from.
+struct GaussGrad {
+    float opac, color[3], scale[3], mean[3];
+    float4 quat;
+};
+
+__device__ __forceinline__ GaussGrad load_gauss_grad(const DbArgs& a, size_t g) {
+    GaussGrad o;
+    o.opac = a.drec[9 * g + 5];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        o.color[e] = a.drec[9 * g + 6 + e];
+        o.scale[e] = a.dscales[3 * g + e];
+        o.mean[e] = a.dmeans[3 * g + e];
+    }
+    o.quat = *reinterpret_cast<const float4*>(a.dquats + 4 * g);
+    return o;
+}
+
+// Gradients of the loss w.r.t. a Gaussian's decoder outputs y: opacity w tanh (zero where the
+// opacity was dropped), colour sigmoid, scale l_v sigmoid (its l_v term added to dlv), unit
+// quaternion.
+__device__ __forceinline__ void dy_opacity(const GaussGrad& g, float w, const float* y, float* dy) {
+    const float th = tanhf(y[0]);
+    dy[0] = w * th > 0.f ? g.opac * w * (1.f - th * th) : 0.f;
+}
+
+__device__ __forceinline__ void dy_color(const GaussGrad& g, const float* y, float* dy) {
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        const float sg = sigm(y[e]);
+        dy[e] = g.color[e] * sg * (1.f - sg);
+    }
+}
+
+__device__ __forceinline__ void dy_cov(const GaussGrad& g, const float (&lvv)[3], const float* y,
+                                       float* dy, float (&dlv)[3]) {
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        const float sg = sigm(y[e]);
+        const float gsc = g.scale[e];
+        dlv[e] += gsc * sg;
+        dy[e] = gsc * lvv[e] * sg * (1.f - sg);
+    }
+    const float n2 = y[3] * y[3] + y[4] * y[4] + y[5] * y[5] + y[6] * y[6];
+    const float inv = 1.0f / sqrtf(n2);
+    const float qn[4] = {y[3] * inv, y[4] * inv, y[5] * inv, y[6] * inv};
+    const float gqa[4] = {g.quat.x, g.quat.y, g.quat.z, g.quat.w};
+    const float dot = qn[0] * gqa[0] + qn[1] * gqa[1] + qn[2] * gqa[2] + qn[3] * gqa[3];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) dy[3 + e] = (gqa[e] - qn[e] * dot) * inv;
+}
+
+// The gradients of decoder m's outputs for Gaussian i of anchor j (row g = r k + i of the
+// Gaussian arrays); with the covariance decoder also the position terms of l_v (dlv) and of the
+// offsets (accumulated in doffs).
 __device__ __forceinline__ void gaussian_dy(const DbArgs& a, int m, size_t g, uint32_t j, int i,
                                             float w, const float (&lvv)[3], const float* y,
                                             float* dy, float (&dlv)[3]) {
+    const GaussGrad gg = load_gauss_grad(a, g);
     if (m == 0) {
-        const float th = tanhf(y[0]);
-        dy[0] = w * th > 0.f ? a.drec[9 * g + 5] * w * (1.f - th * th) : 0.f;
+        dy_opacity(gg, w, y, dy);
     } else if (m == 1) {
-#pragma unroll
-        for (int e = 0; e < 3; ++e) {
-            const float sg = sigm(y[e]);
-            dy[e] = a.drec[9 * g + 6 + e] * sg * (1.f - sg);
-        }
+        dy_color(gg, y, dy);
     } else {
-#pragma unroll
-        for (int e = 0; e < 3; ++e) {
-            const float sg = sigm(y[e]);
-            const float gsc = a.dscales[3 * g + e];
-            dlv[e] += gsc * sg;
-            dy[e] = gsc * lvv[e] * sg * (1.f - sg);
-        }
-        const float n2 = y[3] * y[3] + y[4] * y[4] + y[5] * y[5] + y[6] * y[6];
-        const float inv = 1.0f / sqrtf(n2);
-        const float4 gq = *reinterpret_cast<const float4*>(a.dquats + 4 * g);
-        const float qn[4] = {y[3] * inv, y[4] * inv, y[5] * inv, y[6] * inv};
-        const float gqa[4] = {gq.x, gq.y, gq.z, gq.w};
-        const float dot = qn[0] * gqa[0] + qn[1] * gqa[1] + qn[2] * gqa[2] + qn[3] * gqa[3];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) dy[3 + e] = (gqa[e] - qn[e] * dot) * inv;
+        dy_cov(gg, lvv, y, dy, dlv);
         // positions: mu = x_v + O * l_v
         const float* O = a.offs + ((size_t)j * kK + i) * 3;
 #pragma unroll
         for (int e = 0; e < 3; ++e) {
-            const float gmu = a.dmeans[3 * g + e];
-            a.doffs[((size_t)j * kK + i) * 3 + e] += gmu * lvv[e];
-            dlv[e] += gmu * O[e];
+            a.doffs[((size_t)j * kK + i) * 3 + e] += gg.mean[e] * lvv[e];
+            dlv[e] += gg.mean[e] * O[e];
         }
     }
 }

@@ -231,8 +231,9 @@ __global__ void __launch_bounds__(kDbThreads, 3) decode_bwd_rows(DbArgs a) {
         }
         float* yrow = a.rowY + (size_t)r * kRowY;
         if (cov_half) {
-            yrow[kNOut] = 0.f;
-            yrow[kNOut + 1] = 0.f;
+#pragma unroll
+            for (int e = 0; e < kRowY; ++e)
+                if (row_out(e) < 0) yrow[e] = 0.f;
         }
         const size_t g0 = (size_t)r * kK;
 #pragma unroll 1
@@ -312,7 +313,7 @@ __global__ void __launch_bounds__(kDbThreads, 3) decode_bwd_rows(DbArgs a) {
                 for (int e = 0; e < 7; ++e) {
                     if (e < per) {
                         const int row = out_base(m) + per * i + e;
-                        yrow[row] = dy[e];
+                        yrow[out_row(row)] = dy[e];
                         const float4* wr = reinterpret_cast<const float4*>(sW2 + row * kH);
 #pragma unroll
                         for (int q = 0; q < kH / 4; ++q) {
@@ -393,19 +394,19 @@ __global__ void __launch_bounds__(kDbThreads, 3) decode_bwd_rows(DbArgs a) {
 // 128 -> 49 us; same summation order, same bits.
 constexpr int kWThreads = 256;
 constexpr int kWChunk = 32;
-constexpr int kTilesW2 = (3 + 8 + 18) * (kH / 8);         // row groups of 4 per decoder, 8 columns
+constexpr int kTilesW2 = kRowY / 4 * (kH / 8);           // 3 + 8 + 18 row groups of 4, 8 columns
 constexpr int kTilesW1 = (3 * kH / 8) * (kDin / 4);       // 8 rows, 4 columns
 constexpr int kTiles = kTilesW2 + kTilesW1;               // 224: the last warp sums the biases
 constexpr int kItems1 = kNOut + kNB1;                     // 206 bias sums
 constexpr int kBiasThreads = kWThreads - kTiles;
 static_assert(kTiles % 32 == 0 && kBiasThreads > 0, "whole warps per role");
-static_assert(kK == 10 && kH == 32 && kDin == 36, "block layout of the weight gradients");
+static_assert(kH == 32 && kDin == 36 && kRowCol == 12 && kRowCov == 44 && kRowY == 116,
+              "block layout of the weight gradients");
 
 // Block of the weight gradients owned by thread t < kTiles: four values a and eight values b of
 // an anchor's rows, out[i][j] = sum a_i b_j.  dW2 blocks: a = dy rows row .. row + 3, b = hidden
-// columns col .. col + 7 of decoder dec (the group of rows 8 .. 11 belongs to two decoders and is
-// formed for both; only a decoder's own rows are written).  dW1 blocks: a = inputs col .. col + 3,
-// b = dp rows row .. row + 7.
+// columns col .. col + 7 of its decoder dec (sums over a row's padding are not written).  dW1
+// blocks: a = inputs col .. col + 3, b = dp rows row .. row + 7.
 struct WBlock {
     bool w2;
     int row, col, dec;
@@ -417,7 +418,7 @@ __device__ __forceinline__ WBlock weight_block(int t) {
     if (b.w2) {
         const int rg = t / (kH / 8);
         b.dec = rg < 3 ? 0 : (rg < 11 ? 1 : 2);
-        b.row = rg < 3 ? 4 * rg : (rg < 11 ? 8 + 4 * (rg - 3) : 4 * kK + 4 * (rg - 11));
+        b.row = 4 * rg;
         b.col = 8 * (t % (kH / 8));
     } else {
         const int i = t - kTilesW2;
@@ -527,7 +528,7 @@ __global__ void __launch_bounds__(kWThreads) decode_bwd_weights(DbArgs a) {
                 float s = 0.f;
                 if (item < kNOut) {
 #pragma unroll 8
-                    for (int k = 0; k < kWChunk; ++k) s += sY[k][item];
+                    for (int k = 0; k < kWChunk; ++k) s += sY[k][out_row(item)];
                 } else if (item < kItems1) {
 #pragma unroll 8
                     for (int k = 0; k < kWChunk; ++k) s += sP[k][item - kNOut];
@@ -547,9 +548,8 @@ __global__ void __launch_bounds__(kWThreads) decode_bwd_weights(DbArgs a) {
             for (int j = 0; j < 8; ++j) {
                 const float v = j & 1 ? hi2(acc[i][j / 2]) : lo2(acc[i][j / 2]);
                 if (wb.w2) {
-                    const int row = wb.row + i;
-                    if (row < kNOut && dec_of(row) == wb.dec)
-                        out[kOffW2 + row * kH + wb.col + j] = v;
+                    const int row = row_out(wb.row + i);
+                    if (row >= 0) out[kOffW2 + row * kH + wb.col + j] = v;
                 } else {
                     out[(wb.row + j) * kDin + wb.col + i] = v;
                 }
