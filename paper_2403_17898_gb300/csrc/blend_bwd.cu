@@ -52,7 +52,6 @@ struct __align__(16) BwdSmem {
 };
 
 __device__ __forceinline__ f32x2 as2(float2 v) { return pack2(v.x, v.y); }
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, pack2(-1.f, -1.f), a); }
 
 // Sums the ng parked entries of this warp over its block and adds them to drec.  Lane
 // (part, e) takes entry e, whose record lies at offset `at`, and pixel pairs [part kSlots, ...);

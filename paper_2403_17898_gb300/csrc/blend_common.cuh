@@ -57,12 +57,6 @@ __device__ __forceinline__ uint32_t warp_blocks(const float4& r0, const float4& 
     return m;
 }
 
-__device__ __forceinline__ float rcp(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 // A record as the walks read it (16-byte broadcast loads): the conic scaled and negated so that
 // the walk forms q = -power2 = -log2(e) power >= 0 (negation commutes with rounding: the bits of
 // power2), and the skip bound alpha >= 1/255 <=> q <= qskip.

@@ -6,11 +6,24 @@
 // + C1, A2 = 2 (m3 - m1 my) + C2, B1 = m1^2 + my^2 + C1, B2 = m2 - m1^2 + sy^2 + C2):
 //   dS/dm1 = S (2my/A1 - 2my/A2 - 2m1/B1 + 2m1/B2),  dS/dm2 = -S/B2,  dS/dm3 = 2S/A2,
 // and for the mean SSIM:  d/dx = G*g1 + 2 x (G*g2) + y (G*g3), g_i = dS/dm_i / n.
-// Two tiled passes (moments -> SSIM map and partial maps; blur of the partial maps ->
-// gradient), each staging its tile and halo in shared memory; bound by FP32 instruction issue
-// (11-tap blurs of every moment in both directions).  A training loop that renders against
-// fixed targets can compute the target's two moments once (ogs_ssim_target_stats) and pass
-// them in, so that the forward pass blurs three moments instead of five.
+// Two passes (moments -> SSIM map and partial maps; blur of the partial maps -> gradient).  A
+// training loop that renders against fixed targets can compute the target's two moments once
+// (ogs_ssim_target_stats) and pass them in, so that the forward pass blurs three moments instead
+// of five.
+//
+// Both passes are the same walk: a warp owns a strip of 64 columns (two per lane) and marches
+// down its rows.  A row pair of the inputs (with a kRad halo; zero outside the image: the
+// zero-padded window) passes through a warp-private shared buffer, is blurred horizontally with
+// its two rows packed in one register pair, and enters the vertical blur at once: ten partial
+// sums per moment live in registers and each row adds its tap to all of them while shifting them
+// by one (the shift is the destination of the fused multiply-add), packed over the lane's two
+// columns.  Nothing blurred goes through memory, and no warp waits for another.  Bound by the FP32
+// pipes (66 packed operations per row, two columns and three moments) and the partial maps'
+// traffic.  1080p: forward 57 -> 44 us, backward 54 -> 41 us against 32 x 32 tiles with both blurs
+// staged in shared memory, which spent 250 instructions on a pixel (now 142 and 121); the blurs sum
+// in the same order.  The next row pair is copied asynchronously while the current one is blurred
+// (loads into registers were sunk to their use: 71 and 48 us).  The last strip of the gradient adds
+// the loss, which was a launch of its own.
 #include <cmath>
 
 #include "internal.cuh"
@@ -39,352 +52,298 @@ Win make_window() {
     return g;
 }
 
-// Tiled passes: a CTA owns a kTX x kTY output tile of one channel.  It stages the inputs of
-// the tile plus a kRad halo in shared memory (zero outside the image: the zero-padded window),
-// blurs horizontally into shared memory and vertically into registers.
-constexpr int kTX = 32, kTY = 32;
-constexpr int kHX = kTX + 2 * kRad, kHY = kTY + 2 * kRad;   // 42 x 42 staged inputs
-constexpr int kLossThreads = 256;
+constexpr int kCols = 64;                  // columns of a strip, two per lane
+constexpr int kStripWarps = 2;             // strips (one below the other) per CTA
+constexpr int kSpan = kCols + 2 * kRad;    // 74 input columns
+constexpr int kBufCols = 76;
 
-__device__ __forceinline__ float block_sum(float v, float* red) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane_id() == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    float s = 0.f;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < kLossThreads / 32; ++i) s += red[i];
-    return s;                                       // valid in thread 0
+enum Pass { kMoments3, kMoments5, kGradient, kTargetStats };
+__host__ __device__ constexpr int pass_inputs(Pass p) { return p == kGradient ? 3 : (p == kTargetStats ? 1 : 2); }
+__host__ __device__ constexpr int pass_moments(Pass p) { return p == kMoments5 ? 5 : (p == kTargetStats ? 2 : 3); }
+
+// Sums over the image, zeroed by the call.  In 64 bits: a thousand strips add to each.
+struct LossSums {
+    double ssim, l1;
+    unsigned int done;      // strips whose gradient is finished
+};
+
+struct StripArgs {
+    const float* in[3];     // planes [C][H][W] that are blurred (or whose products are)
+    const float* x;         // kGradient: image and target
+    const float* y;
+    const float* ystat;     // kMoments3: the target's moments [2][C][H][W]
+    float* out;             // partial maps [3][C][H][W] / gradient [C][H][W] / moments [2][C][H][W]
+    LossSums* sums;
+    float* loss;            // kGradient: the loss is added here (may be null)
+    Win g;
+    int H, W, rows;         // rows of a strip
+    int64_t n;              // C H W
+    float inv_n, lam;
+    unsigned int strips;    // strips of the launch
+    int vec;                // W even and every plane 8-byte aligned: a lane's columns as one vector
+};
+
+// Asynchronous 4- and 8-byte copies global -> shared; bytes = 0 reads nothing and writes zeros.
+__device__ __forceinline__ void copy4(float* dst, const float* src, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void copy8(float* dst, const float* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ f32x2 shared2(const float* p) {
+    const float2 v = *reinterpret_cast<const float2*>(p);
+    return pack2(v.x, v.y);
 }
 
-// Register-blocked 11-tap blurs: a thread produces kRun consecutive outputs along the blur
-// direction from kRun + 10 loaded inputs (each input loaded once instead of once per tap).
-constexpr int kRun = 4;
-constexpr int kSpan = kRun + kWin - 1;                     // 14 inputs per run
-constexpr int kHRuns = kHY * (kTX / kRun);                 // 42 rows x 8 runs = 336
-constexpr int kVRuns = kTX * (kTY / kRun);                 // 32 columns x 8 runs = 256
+// the lane's two columns of a row, packed (in1: the second lies in the image)
+__device__ __forceinline__ void store2(float* p, f32x2 v, bool in1, int vec) {
+    if (vec) {
+        *reinterpret_cast<float2*>(p) = make_float2(lo2(v), hi2(v));
+    } else {
+        p[0] = lo2(v);
+        if (in1) p[1] = hi2(v);
+    }
+}
+__device__ __forceinline__ f32x2 both(float v) { return pack2(v, v); }
+// reciprocals, a few ulp: four of them in place of seven divisions per pixel
+__device__ __forceinline__ f32x2 rcp2(f32x2 v) { return pack2(rcp(lo2(v)), rcp(hi2(v))); }
 
-// pass 1: the blurred moments -> SSIM map (summed) and the three partial maps
-// gp_i = dS/dm_i / n for the backward.  The five moments are G*x, G*y, G*x^2, G*y^2, G*xy;
-// with kCached the target's two (G*y, G*y^2) come precomputed in ystat[2][C][H][W] (they do
-// not change between training steps) and only three are blurred here.
-template <bool kCached>
-__global__ void __launch_bounds__(kLossThreads) ssim_fwd(const float* __restrict__ x,
-                                                         const float* __restrict__ y, int H, int W,
-                                                         Win g, float inv_n,
-                                                         float* __restrict__ gp, int64_t n,
-                                                         float* __restrict__ ssim_sum,
-                                                         const float* __restrict__ ystat) {
-    constexpr int kM = kCached ? 3 : 5;           // moments blurred here: x, [y], x^2, [y^2], xy
-    __shared__ float sx[kHY][kHX + 1];
-    __shared__ float sy[kHY][kHX + 1];
-    __shared__ float hs[kM][kHY][kTX + 1];
-    __shared__ float red[kLossThreads / 32];
-    const int c = blockIdx.z;
-    const int x0 = blockIdx.x * kTX - kRad, y0 = blockIdx.y * kTY - kRad;
-    const int64_t plane = (int64_t)c * H * W;
-    {
-        // 6 rows of 42 per pass, 7 passes; all loads issued before any store (threads 252..255
-        // idle)
-        constexpr int kRowsPer = kLossThreads / kHX, kPasses = (kHY + kRowsPer - 1) / kRowsPer;
-        const int q = threadIdx.x % kHX, r0 = threadIdx.x / kHX;
-        const bool act = threadIdx.x < kRowsPer * kHX;
-        float vx[kPasses], vy[kPasses];
+// The lane's two pixels of the forward pass from their moments: the SSIM values and the partial
+// maps gp_i = dS/dm_i / n.
+__device__ __forceinline__ f32x2 ssim_pixels(f32x2 mx, f32x2 my, f32x2 exx, f32x2 eyy, f32x2 exy,
+                                             float inv_n, f32x2& g0, f32x2& g1, f32x2& g2) {
+    const f32x2 nx = mul2(mx, both(-1.f)), ny = mul2(my, both(-1.f));
+    const f32x2 vx = fma2(nx, mx, exx), vy = fma2(ny, my, eyy), vxy = fma2(nx, my, exy);
+    const f32x2 A1 = fma2(add2(mx, mx), my, both(kC1)), A2 = add2(add2(vxy, vxy), both(kC2));
+    const f32x2 B1 = add2(fma2(mx, mx, mul2(my, my)), both(kC1));
+    const f32x2 B2 = add2(add2(vx, vy), both(kC2));
+    const f32x2 iA1 = rcp2(A1), iA2 = rcp2(A2), iB1 = rcp2(B1), iB2 = rcp2(B2);
+    const f32x2 S = mul2(mul2(mul2(A1, A2), iB1), iB2);
+    const f32x2 sS = mul2(S, both(inv_n)), s2 = add2(sS, sS);
+    g0 = mul2(s2, fma2(my, sub2(iA1, iA2), mul2(mx, sub2(iB2, iB1))));
+    g1 = mul2(mul2(sS, both(-1.f)), iB2);
+    g2 = mul2(s2, iA2);
+    return S;
+}
+
+// kMoments: moments -> SSIM map (summed) and the three partial maps.  The five moments are G*x,
+// G*y, G*x^2, G*y^2, G*xy; kMoments3 takes the target's two from ystat.
+// kGradient: blur of the partial maps -> dSSIM/dx = G*gp0 + 2 x (G*gp1) + y (G*gp2);
+// out = (1 - lam) sign(x - y) / n - lam dSSIM/dx, and the L1 sum.
+// kTargetStats: G*y and G*y^2.
+// CTAs per SM that the registers allow (kMoments5: five).  More CTAs at 128 registers recompute what
+// they cannot keep: 8 CTAs 50 and 48 us.
+constexpr int kCtas = 6;
+template <Pass kPass>
+__global__ void __launch_bounds__(32 * kStripWarps, kPass == kMoments5 ? 5 : kCtas) ssim_strip(StripArgs a) {
+    constexpr int kIn = pass_inputs(kPass), kM = pass_moments(kPass);
+    constexpr bool kExtra = kPass == kMoments3 || kPass == kGradient;
+    // a row pair of the inputs, the two rows of a column together; what its epilogue reads
+    __shared__ __align__(16) float2 s_buf[kStripWarps][2][kIn][kBufCols];
+    __shared__ __align__(16) float s_ext[kStripWarps][2][kExtra ? 4 * kCols : 1];
+    pdl_wait();
+    pdl_trigger();
+    const int lane = (int)lane_id(), w = threadIdx.x >> 5;
+    const int y0 = (int)(blockIdx.y * kStripWarps + w) * a.rows;
+    if (y0 >= a.H) return;                                 // whole warps; no block barrier below
+    const int y1 = min(y0 + a.rows, a.H);
+    const int xs = (int)blockIdx.x * kCols;
+    const int64_t plane = (int64_t)blockIdx.z * a.H * a.W;
+    const int gx = xs + 2 * lane;                          // this lane's output columns gx, gx + 1
+    const bool in0 = gx < a.W, in1 = gx + 1 < a.W;
+    f32x2 wt[kWin];                                        // the window is symmetric: six pairs
 #pragma unroll
-        for (int k = 0; k < kPasses; ++k) {
-            const int gy = y0 + r0 + kRowsPer * k, gx = x0 + q;
-            const bool in = act && r0 + kRowsPer * k < kHY && gx >= 0 && gx < W && gy >= 0 && gy < H;
-            const int64_t i = plane + (int64_t)gy * W + gx;
-            vx[k] = in ? x[i] : 0.f;
-            vy[k] = in ? y[i] : 0.f;
-        }
+    for (int k = 0; k < kWin; ++k) wt[k] = pack2(a.g.w[k < kRad ? k : kWin - 1 - k],
+                                                 a.g.w[k < kRad ? k : kWin - 1 - k]);
+    int cin[3];                                            // bytes of input column lane + 32 q
 #pragma unroll
-        for (int k = 0; k < kPasses; ++k) {
-            if (act && r0 + kRowsPer * k < kHY) {
-                sx[r0 + kRowsPer * k][q] = vx[k];
-                sy[r0 + kRowsPer * k][q] = vy[k];
-            }
-        }
+    for (int q = 0; q < 3; ++q) {
+        const int col = lane + 32 * q, cx = xs - kRad + col;
+        cin[q] = col < kSpan && cx >= 0 && cx < a.W ? 4 : 0;
     }
-    __syncthreads();
-    for (int e = threadIdx.x; e < kHRuns; e += kLossThreads) {
-        const int r = e >> 3, q0 = (e & 7) * kRun;
-        float u[kSpan], v[kSpan];
+    const int nr = y1 - y0 + 2 * kRad;                     // input rows of the strip
+    // the lane's first input column in the next row to be copied, and its output columns in the
+    // epilogue's operands of the output row that the copied row completes
+    const int64_t at = plane + (int64_t)(y0 - kRad) * a.W + xs - kRad + lane;
+    const float* pin[kIn];
 #pragma unroll
-        for (int k = 0; k < kSpan; ++k) { u[k] = sx[r][q0 + k]; v[k] = sy[r][q0 + k]; }
-        float acc[kM][kRun];
+    for (int j = 0; j < kIn; ++j) pin[j] = a.in[j] + at;
+    const int64_t o = plane + (int64_t)(y0 - 2 * kRad) * a.W + gx;
+    const float* ext[2] = {(kPass == kGradient ? a.x : a.ystat) + o,
+                           (kPass == kGradient ? a.y : a.ystat + a.n) + o};
+    // copies input rows r, r + 1 of the strip into buffer b, zero outside the image, with the
+    // epilogue's operands of output rows r - 2 kRad, r + 1 - 2 kRad
+    auto fetch = [&](int r, int b) {
+        float* buf = reinterpret_cast<float*>(&s_buf[w][b][0][lane]);
+        float* eb = &s_ext[w][b][kExtra ? 2 * lane : 0];
 #pragma unroll
-        for (int t = 0; t < kRun; ++t)
+        for (int h = 0; h < 2; ++h) {
+            const bool rin = (unsigned)(y0 - kRad + r + h) < (unsigned)a.H;
 #pragma unroll
-            for (int j = 0; j < kM; ++j) acc[j][t] = 0.f;
+            for (int q = 0; q < 3; ++q) {
+                const int bytes = rin ? cin[q] : 0;
+                if (q < 2 || lane < kBufCols - 64)
 #pragma unroll
-        for (int k = 0; k < kSpan; ++k) {
-            // channel order: x, x^2, xy (cached) or x, y, x^2, y^2, xy
-            float ch[kM];
-            if (kCached) {
-                ch[0] = u[k];
-                ch[1] = u[k] * u[k];
-                ch[kM - 1] = u[k] * v[k];
-            } else {
-                ch[0] = u[k];
-                ch[1] = v[k];
-                ch[2] = u[k] * u[k];
-                ch[3] = v[k] * v[k];
-                ch[kM - 1] = u[k] * v[k];
+                    for (int j = 0; j < kIn; ++j)
+                        copy4(buf + 2 * (kBufCols * j + 32 * q) + h, pin[j] + 32 * q, bytes);
             }
 #pragma unroll
-            for (int t = 0; t < kRun; ++t) {
-                const int tap = k - t;
-                if (tap < 0 || tap >= kWin) continue;
-                const float w = g.w[tap];
+            for (int j = 0; j < kIn; ++j) pin[j] += a.W;
+            if (kExtra) {
+                if (r >= 2 * kRad && r + h < nr && in0) {
 #pragma unroll
-                for (int j = 0; j < kM; ++j) acc[j][t] = fmaf(w, ch[j], acc[j][t]);
+                    for (int j = 0; j < 2; ++j) {
+                        float* d = eb + (2 * j + h) * kCols;
+                        if (a.vec) {
+                            copy8(d, ext[j]);
+                        } else {
+                            copy4(d, ext[j], 4);
+                            copy4(d + 1, ext[j] + 1, in1 ? 4 : 0);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) ext[j] += a.W;
             }
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    f32x2 acc[kM][kWin - 1];
 #pragma unroll
-        for (int t = 0; t < kRun; ++t)
+    for (int j = 0; j < kM; ++j)
 #pragma unroll
-            for (int j = 0; j < kM; ++j) hs[j][r][q0 + t] = acc[j][t];
-    }
-    __syncthreads();
+        for (int k = 0; k < kWin - 1; ++k) acc[j][k] = 0;
     float local = 0.f;
-    {
-        const int qc = threadIdx.x & 31, r0 = (threadIdx.x >> 5) * kRun;   // one run per thread
-        float m[kM][kRun];
+    fetch(0, 0);
+    float* out[3] = {a.out + o, a.out + a.n + o, a.out + 2 * a.n + o};
+    for (int r = 0; r < nr; r += 2) {
+        const int b = (r >> 1) & 1;
+        __syncwarp();                                      // the other buffer has been read
+        if (r + 2 < nr) fetch(r + 2, b ^ 1);
+        else asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();                                      // every lane's copies have landed
+        const float2(*buf)[kBufCols] = s_buf[w][b];
+        // horizontal blur of both rows (packed) for the lane's two columns
+        f32x2 hb[kM][2];
 #pragma unroll
-        for (int t = 0; t < kRun; ++t)
+        for (int j = 0; j < kM; ++j) hb[j][0] = hb[j][1] = 0;
 #pragma unroll
-            for (int j = 0; j < kM; ++j) m[j][t] = 0.f;
+        for (int k2 = 0; k2 < kWin + 1; k2 += 2) {
+            float4 v4[kIn];
 #pragma unroll
-        for (int k = 0; k < kSpan; ++k) {
-            float hv[kM];
+            for (int j = 0; j < kIn; ++j)
+                v4[j] = *reinterpret_cast<const float4*>(&buf[j][2 * lane + k2]);
 #pragma unroll
-            for (int j = 0; j < kM; ++j) hv[j] = hs[j][r0 + k][qc];
+            for (int u = 0; u < 2; ++u) {
+                const int k = k2 + u;
+                f32x2 in[kIn], ch[kM];
 #pragma unroll
-            for (int t = 0; t < kRun; ++t) {
-                const int tap = k - t;
-                if (tap < 0 || tap >= kWin) continue;
-                const float w = g.w[tap];
+                for (int j = 0; j < kIn; ++j)
+                    in[j] = u ? pack2(v4[j].z, v4[j].w) : pack2(v4[j].x, v4[j].y);
+                if (kPass == kMoments3) {
+                    ch[0] = in[0]; ch[1] = mul2(in[0], in[0]); ch[2] = mul2(in[0], in[1]);
+                } else if (kPass == kMoments5) {
+                    ch[0] = in[0]; ch[1] = in[1]; ch[2] = mul2(in[0], in[0]);
+                    ch[kM - 2] = mul2(in[1], in[1]); ch[kM - 1] = mul2(in[0], in[1]);
+                } else if (kPass == kTargetStats) {
+                    ch[0] = in[0]; ch[1] = mul2(in[0], in[0]);
+                } else {
 #pragma unroll
-                for (int j = 0; j < kM; ++j) m[j][t] = fmaf(w, hv[j], m[j][t]);
+                    for (int j = 0; j < kM; ++j) ch[j] = in[j < kIn ? j : 0];
+                }
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    const int tap = k - t;
+                    if (tap < 0 || tap >= kWin) continue;
+#pragma unroll
+                    for (int j = 0; j < kM; ++j) hb[j][t] = fma2(wt[tap], ch[j], hb[j][t]);
+                }
             }
         }
-        const int gx = x0 + kRad + qc;
+        // vertical blur, one row at a time, both columns packed
 #pragma unroll
-        for (int t = 0; t < kRun; ++t) {
-            const int gy = y0 + kRad + r0 + t;
-            if (gx >= W || gy >= H) continue;
-            const int64_t i = plane + (int64_t)gy * W + gx;
-            float mx, my, exx, eyy, exy;
-            if (kCached) {
-                mx = m[0][t]; exx = m[1][t]; exy = m[2][t];
-                my = ystat[i]; eyy = ystat[n + i];
+        for (int h = 0; h < 2; ++h) {
+            f32x2 m[kM];
+#pragma unroll
+            for (int j = 0; j < kM; ++j) {
+                const f32x2 v = h ? pack2(hi2(hb[j][0]), hi2(hb[j][1]))
+                                  : pack2(lo2(hb[j][0]), lo2(hb[j][1]));
+                m[j] = fma2(wt[kWin - 1], v, acc[j][0]);
+#pragma unroll
+                for (int k = 0; k < kWin - 2; ++k) acc[j][k] = fma2(wt[kWin - 2 - k], v, acc[j][k + 1]);
+                acc[j][kWin - 2] = fma2(wt[0], v, 0);
+            }
+            const bool write = r >= 2 * kRad && r + h < nr && in0;
+            f32x2 e0 = 0, e1 = 0;
+            if (kExtra && write) {
+                e0 = shared2(&s_ext[w][b][kExtra ? h * kCols + 2 * lane : 0]);
+                e1 = shared2(&s_ext[w][b][kExtra ? (2 + h) * kCols + 2 * lane : 0]);
+            }
+            if (!write) {
+            } else if (kPass == kTargetStats) {
+                store2(out[0], m[0], in1, a.vec);
+                store2(out[1], m[1], in1, a.vec);
+            } else if (kPass == kGradient) {
+                const f32x2 df = sub2(e0, e1);
+                const float d0 = lo2(df), d1 = hi2(df);
+                local += fabsf(d0) + (in1 ? fabsf(d1) : 0.f);
+                const f32x2 sgn = pack2(d0 > 0.f ? a.inv_n : (d0 < 0.f ? -a.inv_n : 0.f),
+                                        d1 > 0.f ? a.inv_n : (d1 < 0.f ? -a.inv_n : 0.f));
+                const f32x2 dssim = fma2(e1, m[kM - 1], fma2(add2(e0, e0), m[1], m[0]));
+                store2(out[0], fma2(both(-a.lam), dssim, mul2(both(1.f - a.lam), sgn)), in1, a.vec);
             } else {
-                mx = m[0][t]; my = m[1][t]; exx = m[2][t]; eyy = m[3][t]; exy = m[4][t];
+                const bool c3 = kPass == kMoments3;
+                f32x2 g0, g1, g2;
+                const f32x2 S = ssim_pixels(m[0], c3 ? e0 : m[1], c3 ? m[1] : m[2 % kM],
+                                            c3 ? e1 : m[3 % kM], m[kM - 1], a.inv_n, g0, g1, g2);
+                local += lo2(S) + (in1 ? hi2(S) : 0.f);
+                store2(out[0], g0, in1, a.vec);
+                store2(out[1], g1, in1, a.vec);
+                store2(out[2], g2, in1, a.vec);
             }
-            const float vx = exx - mx * mx, vy = eyy - my * my, vxy = exy - mx * my;
-            const float A1 = 2.f * mx * my + kC1, A2 = 2.f * vxy + kC2;
-            const float B1 = mx * mx + my * my + kC1, B2 = vx + vy + kC2;
-            // four fast reciprocals (a few ulp) in place of seven divisions: the epilogue
-            // would otherwise cost as much as the blurs
-            const float iA1 = __fdividef(1.f, A1), iA2 = __fdividef(1.f, A2);
-            const float iB1 = __fdividef(1.f, B1), iB2 = __fdividef(1.f, B2);
-            const float S = A1 * A2 * iB1 * iB2;
-            local += S;
-            const float sS = S * inv_n;
-            gp[i] = 2.f * sS * (my * (iA1 - iA2) + mx * (iB2 - iB1));
-            gp[n + i] = -sS * iB2;
-            gp[2 * n + i] = 2.f * sS * iA2;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) out[j] += a.W;
         }
     }
-    const float s = block_sum(local, red);
-    if (threadIdx.x == 0) atomicAdd(ssim_sum, s);
-}
-
-// pass 2: blur of the partial maps -> dSSIM/dx = G*gp0 + 2 x (G*gp1) + y (G*gp2);
-// dimg = (1 - lam) sign(x - y) / n - lam dSSIM/dx, and the L1 sum
-__global__ void __launch_bounds__(kLossThreads) ssim_bwd(const float* __restrict__ gp,
-                                                         const float* __restrict__ x,
-                                                         const float* __restrict__ y, int H, int W,
-                                                         Win g, float lam, float inv_n, int64_t n,
-                                                         float* __restrict__ dimg,
-                                                         float* __restrict__ l1_sum) {
-    __shared__ float sg[3][kHY][kHX + 1];
-    __shared__ float hs[3][kHY][kTX + 1];
-    __shared__ float red[kLossThreads / 32];
-    const int c = blockIdx.z;
-    const int x0 = blockIdx.x * kTX - kRad, y0 = blockIdx.y * kTY - kRad;
-    const int64_t plane = (int64_t)c * H * W;
-    {
-        constexpr int kRowsPer = kLossThreads / kHX, kPasses = (kHY + kRowsPer - 1) / kRowsPer;
-        const int q = threadIdx.x % kHX, r0 = threadIdx.x / kHX;
-        const bool act = threadIdx.x < kRowsPer * kHX;
-        float v0[kPasses], v1[kPasses], v2[kPasses];
+    if (kPass != kTargetStats) {
 #pragma unroll
-        for (int k = 0; k < kPasses; ++k) {
-            const int gy = y0 + r0 + kRowsPer * k, gx = x0 + q;
-            const bool in = act && r0 + kRowsPer * k < kHY && gx >= 0 && gx < W && gy >= 0 && gy < H;
-            const int64_t i = plane + (int64_t)gy * W + gx;
-            v0[k] = in ? gp[i] : 0.f;
-            v1[k] = in ? gp[n + i] : 0.f;
-            v2[k] = in ? gp[2 * n + i] : 0.f;
-        }
-#pragma unroll
-        for (int k = 0; k < kPasses; ++k) {
-            if (act && r0 + kRowsPer * k < kHY) {
-                sg[0][r0 + kRowsPer * k][q] = v0[k];
-                sg[1][r0 + kRowsPer * k][q] = v1[k];
-                sg[2][r0 + kRowsPer * k][q] = v2[k];
+        for (int o = 16; o > 0; o >>= 1) local += __shfl_xor_sync(0xffffffffu, local, o);
+        if (lane == 0) {
+            atomicAdd(kPass == kGradient ? &a.sums->l1 : &a.sums->ssim, (double)local);
+            if (kPass == kGradient && a.loss) {
+                // the last strip: loss = (1 - lam) * mean |x - y| + lam * (1 - mean SSIM)
+                __threadfence();
+                if (atomicAdd(&a.sums->done, 1u) == a.strips - 1) {
+                    __threadfence();
+                    const double l1 = *(volatile double*)&a.sums->l1;
+                    const double ssim = *(volatile double*)&a.sums->ssim, n = (double)a.n;
+                    *a.loss += (float)((1.0 - a.lam) * l1 / n + a.lam * (1.0 - ssim / n));
+                }
             }
         }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < kHRuns; e += kLossThreads) {
-        const int r = e >> 3, q0 = (e & 7) * kRun;
-        float acc[3][kRun];
-#pragma unroll
-        for (int t = 0; t < kRun; ++t)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) acc[j][t] = 0.f;
-#pragma unroll
-        for (int k = 0; k < kSpan; ++k) {
-            float gv[3];
-#pragma unroll
-            for (int j = 0; j < 3; ++j) gv[j] = sg[j][r][q0 + k];
-#pragma unroll
-            for (int t = 0; t < kRun; ++t) {
-                const int tap = k - t;
-                if (tap < 0 || tap >= kWin) continue;
-                const float w = g.w[tap];
-#pragma unroll
-                for (int j = 0; j < 3; ++j) acc[j][t] = fmaf(w, gv[j], acc[j][t]);
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < kRun; ++t)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) hs[j][r][q0 + t] = acc[j][t];
-    }
-    __syncthreads();
-    float local = 0.f;
-    {
-        const int qc = threadIdx.x & 31, r0 = (threadIdx.x >> 5) * kRun;
-        const int gx = x0 + kRad + qc;
-        float xs[kRun], ys[kRun];                 // loaded before the blur, used after it
-#pragma unroll
-        for (int t = 0; t < kRun; ++t) {
-            const int gy = y0 + kRad + r0 + t;
-            const bool in = gx < W && gy < H;
-            const int64_t i = plane + (int64_t)gy * W + gx;
-            xs[t] = in ? x[i] : 0.f;
-            ys[t] = in ? y[i] : 0.f;
-        }
-        float m[3][kRun];
-#pragma unroll
-        for (int t = 0; t < kRun; ++t)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) m[j][t] = 0.f;
-#pragma unroll
-        for (int k = 0; k < kSpan; ++k) {
-            float hv[3];
-#pragma unroll
-            for (int j = 0; j < 3; ++j) hv[j] = hs[j][r0 + k][qc];
-#pragma unroll
-            for (int t = 0; t < kRun; ++t) {
-                const int tap = k - t;
-                if (tap < 0 || tap >= kWin) continue;
-                const float w = g.w[tap];
-#pragma unroll
-                for (int j = 0; j < 3; ++j) m[j][t] = fmaf(w, hv[j], m[j][t]);
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < kRun; ++t) {
-            const int gy = y0 + kRad + r0 + t;
-            if (gx >= W || gy >= H) continue;
-            const int64_t i = plane + (int64_t)gy * W + gx;
-            const float xi = xs[t], yi = ys[t];
-            const float dssim = m[0][t] + 2.f * xi * m[1][t] + yi * m[2][t];
-            const float df = xi - yi;
-            local += fabsf(df);
-            const float sgn = df > 0.f ? inv_n : (df < 0.f ? -inv_n : 0.f);
-            dimg[i] = (1.f - lam) * sgn - lam * dssim;
-        }
-    }
-    const float s = block_sum(local, red);
-    if (threadIdx.x == 0) atomicAdd(l1_sum, s);
-}
-
-// The target's two window moments G*y and G*y^2 (zero padded), written to ystat[2][C][H][W]:
-// the same tiling and blur order as ssim_fwd, so the cached form uses the same values.
-__global__ void __launch_bounds__(kLossThreads) ssim_target_stats(const float* __restrict__ y,
-                                                                  int H, int W, Win g, int64_t n,
-                                                                  float* __restrict__ ystat) {
-    __shared__ float sy[kHY][kHX + 1];
-    __shared__ float hs[2][kHY][kTX + 1];
-    const int c = blockIdx.z;
-    const int x0 = blockIdx.x * kTX - kRad, y0 = blockIdx.y * kTY - kRad;
-    const int64_t plane = (int64_t)c * H * W;
-    for (int e = threadIdx.x; e < kHY * kHX; e += kLossThreads) {
-        const int r = e / kHX, q = e % kHX;
-        const int gy = y0 + r, gx = x0 + q;
-        const bool in = gx >= 0 && gx < W && gy >= 0 && gy < H;
-        sy[r][q] = in ? y[plane + (int64_t)gy * W + gx] : 0.f;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < kHRuns; e += kLossThreads) {
-        const int r = e >> 3, q0 = (e & 7) * kRun;
-        float acc[2][kRun];
-#pragma unroll
-        for (int t = 0; t < kRun; ++t) acc[0][t] = acc[1][t] = 0.f;
-#pragma unroll
-        for (int k = 0; k < kSpan; ++k) {
-            const float v = sy[r][q0 + k], vv = v * v;
-#pragma unroll
-            for (int t = 0; t < kRun; ++t) {
-                const int tap = k - t;
-                if (tap < 0 || tap >= kWin) continue;
-                acc[0][t] = fmaf(g.w[tap], v, acc[0][t]);
-                acc[1][t] = fmaf(g.w[tap], vv, acc[1][t]);
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < kRun; ++t) {
-            hs[0][r][q0 + t] = acc[0][t];
-            hs[1][r][q0 + t] = acc[1][t];
-        }
-    }
-    __syncthreads();
-    const int qc = threadIdx.x & 31, r0 = (threadIdx.x >> 5) * kRun;
-    float m[2][kRun];
-#pragma unroll
-    for (int t = 0; t < kRun; ++t) m[0][t] = m[1][t] = 0.f;
-#pragma unroll
-    for (int k = 0; k < kSpan; ++k) {
-        const float h0 = hs[0][r0 + k][qc], h1 = hs[1][r0 + k][qc];
-#pragma unroll
-        for (int t = 0; t < kRun; ++t) {
-            const int tap = k - t;
-            if (tap < 0 || tap >= kWin) continue;
-            m[0][t] = fmaf(g.w[tap], h0, m[0][t]);
-            m[1][t] = fmaf(g.w[tap], h1, m[1][t]);
-        }
-    }
-    const int gx = x0 + kRad + qc;
-#pragma unroll
-    for (int t = 0; t < kRun; ++t) {
-        const int gy = y0 + kRad + r0 + t;
-        if (gx >= W || gy >= H) continue;
-        const int64_t i = plane + (int64_t)gy * W + gx;
-        ystat[i] = m[0][t];
-        ystat[n + i] = m[1][t];
     }
 }
 
-// loss = (1 - lam) * l1_sum / n + lam * (1 - ssim_sum / n), added to *loss
-__global__ void combine_loss(const float* sums, int64_t n, float lam, float* loss) {
-    if (threadIdx.x == 0 && blockIdx.x == 0)
-        *loss += (1.f - lam) * sums[1] / (float)n + lam * (1.f - sums[0] / (float)n);
+// Rows per strip: as many strips as fit the SMs at once, since the ten halo rows of a strip are
+// blurred twice and a second wave of CTAs would double the time (1080p, 12 strips' warps per SM:
+// 54 rows; 900 CTAs in one wave).  A small image gets strips of as few rows as a pair: its time is
+// one strip's, and twelve rows take less than eighteen (strips of at least eight rows lost 2.5 us of
+// 27 on a 0.2-megapixel image against the tiled form).
+constexpr int kMinRows = 2;
+
+template <Pass kPass>
+void launch_strips(StripArgs a, int C, cudaStream_t st) {
+    const int cols = (a.W + kCols - 1) / kCols;
+    int64_t ny = (int64_t)kSmCount * kCtas / ((int64_t)cols * C);
+    if (ny < 1) ny = 1;
+    const int64_t rows = (a.H + ny * kStripWarps - 1) / (ny * kStripWarps);
+    a.rows = (int)(rows < kMinRows ? kMinRows : (rows + 1) / 2 * 2);
+    ny = (a.H + (int64_t)a.rows * kStripWarps - 1) / ((int64_t)a.rows * kStripWarps);
+    a.strips = (unsigned)((a.H + a.rows - 1) / a.rows) * (unsigned)cols * (unsigned)C;
+    launch_pdl(ssim_strip<kPass>, dim3(cols, (unsigned)ny, C), dim3(32 * kStripWarps), 0, st, a);
 }
 
 }  // namespace
@@ -393,15 +352,20 @@ __global__ void combine_loss(const float* sums, int64_t n, float lam, float* los
 using namespace ogs;
 
 extern "C" size_t ogs_loss_l1_ssim_scratch_bytes(int32_t C, int32_t H, int32_t W) {
-    return sizeof(float) * ((size_t)3 * C * H * W + 4) + 512;
+    return sizeof(float) * ((size_t)3 * C * H * W + 4) + 512;   // maps, sums, alignment
 }
 
 extern "C" ogs_status ogs_ssim_target_stats(const float* target, int32_t C, int32_t H,
                                             int32_t W, float* ystat, void* stream) {
     if (!target || !ystat || C <= 0 || H <= 0 || W <= 0) return OGS_ERR_ARG;
-    const dim3 grid((W + kTX - 1) / kTX, (H + kTY - 1) / kTY, C);
-    ssim_target_stats<<<grid, kLossThreads, 0, (cudaStream_t)stream>>>(
-        target, H, W, make_window(), (int64_t)C * H * W, ystat);
+    StripArgs a = {};
+    a.in[0] = target;
+    a.out = ystat;
+    a.g = make_window();
+    a.H = H; a.W = W;
+    a.n = (int64_t)C * H * W;
+    a.vec = W % 2 == 0 && aligned(ystat, 8);
+    launch_strips<kTargetStats>(a, C, (cudaStream_t)stream);
     return launch_status();
 }
 
@@ -417,19 +381,28 @@ extern "C" ogs_status ogs_loss_l1_ssim(const float* img, const float* target, in
     const int64_t n = (int64_t)C * H * W;
     Carver cv(scratch);
     float* gp = cv.take<float>(3 * n);
-    float* sums = cv.take<float>(4);
-    const Win g = make_window();
-    if (cudaMemsetAsync(sums, 0, 4 * sizeof(float), st) != cudaSuccess) return OGS_ERR_CUDA;
-    const dim3 grid((W + kTX - 1) / kTX, (H + kTY - 1) / kTY, C);
-    const float inv_n = 1.0f / (float)n;
-    if (target_stats)
-        ssim_fwd<true><<<grid, kLossThreads, 0, st>>>(img, target, H, W, g, inv_n, gp, n, sums,
-                                                      target_stats);
-    else
-        ssim_fwd<false><<<grid, kLossThreads, 0, st>>>(img, target, H, W, g, inv_n, gp, n, sums,
-                                                       nullptr);
-    ssim_bwd<<<grid, kLossThreads, 0, st>>>(gp, img, target, H, W, g, lambda, inv_n, n, dimg,
-                                            sums + 1);
-    if (loss) combine_loss<<<1, 32, 0, st>>>(sums, n, lambda, loss);
+    LossSums* sums = cv.take<LossSums>(1);
+    if (cudaMemsetAsync(sums, 0, sizeof(LossSums), st) != cudaSuccess) return OGS_ERR_CUDA;
+    StripArgs a = {};
+    a.in[0] = img;
+    a.in[1] = target;
+    a.ystat = target_stats;
+    a.out = gp;
+    a.sums = sums;
+    a.g = make_window();
+    a.H = H; a.W = W;
+    a.n = n;
+    a.inv_n = 1.0f / (float)n;
+    a.lam = lambda;
+    a.vec = W % 2 == 0 && aligned(img, 8) && aligned(target, 8) && aligned(dimg, 8) &&
+            aligned(target_stats, 8);
+    if (target_stats) launch_strips<kMoments3>(a, C, st);
+    else launch_strips<kMoments5>(a, C, st);
+    for (int j = 0; j < 3; ++j) a.in[j] = gp + j * n;
+    a.x = img;
+    a.y = target;
+    a.out = dimg;
+    a.loss = loss;
+    launch_strips<kGradient>(a, C, st);
     return launch_status();
 }
