@@ -118,6 +118,42 @@ __device__ __forceinline__ ProjOut project_one(const Cam& c, float m0, float m1,
 // lane, and rectangles of more than kOwnTiles tiles by the whole warp.
 constexpr uint32_t kOwnTiles = 8;
 
+// Row and column of tile i of a rectangle of width w and n tiles (row-major), without an integer
+// division per tile: i / w by a product with 1 / w.  With n <= 2^20 the quotient (i + 1/2) / w lies
+// at least 1 / (2 w) from a whole number and below n / w, so its relative error of 2^-22 cannot
+// cross one; larger rectangles divide.  (1M Gaussians with 3.7 tiles each: projection with tile
+// counts 67 -> 58 us; the small rectangles walk their rows instead of dividing.)
+struct RectRows {
+    uint32_t w;
+    float inv;
+    bool fast;
+    __device__ __forceinline__ RectRows(uint32_t w_, uint32_t n) {
+        w = w_;
+        inv = __frcp_rn((float)w_);
+        fast = n <= (1u << 20);
+    }
+    __device__ __forceinline__ uint32_t row(uint32_t i) const {
+        return fast ? (uint32_t)(((float)i + 0.5f) * inv) : i / w;
+    }
+};
+
+// Calls f(tile, k) for the tiles of a small rectangle (ntiles <= kOwnTiles) after its first, in
+// order: k = 1 .. ntiles - 1, walked row by row.
+template <class F>
+__device__ __forceinline__ void for_own_tiles(uint32_t t0, uint32_t w, uint32_t ntiles, int gx, F f) {
+    uint32_t kx = 0, t = t0;
+#pragma unroll
+    for (uint32_t i = 1; i < kOwnTiles; ++i) {
+        if (++kx == w) {
+            kx = 0;
+            t += (uint32_t)gx - w + 1;
+        } else {
+            ++t;
+        }
+        if (i < ntiles) f(t, i);
+    }
+}
+
 __device__ __forceinline__ void count_tiles(uint32_t* tc, int gx, uint2 rc, uint32_t ntiles) {
     const uint32_t x0 = rc.x & 0xFFFFu, y0 = rc.x >> 16, x1 = rc.y & 0xFFFFu;
     const uint32_t w = x1 - x0;
@@ -125,8 +161,7 @@ __device__ __forceinline__ void count_tiles(uint32_t* tc, int gx, uint2 rc, uint
     const uint32_t t0 = own ? y0 * (uint32_t)gx + x0 : 0xFFFFFFFFu;
     const uint32_t peers = __match_any_sync(0xffffffffu, t0);
     if (own && lane_id() == (uint32_t)(__ffs(peers) - 1)) atomicAdd(tc + t0, (uint32_t)__popc(peers));
-    if (own)
-        for (uint32_t i = 1; i < ntiles; ++i) atomicAdd(tc + (y0 + i / w) * (uint32_t)gx + x0 + i % w, 1u);
+    if (own) for_own_tiles(t0, w, ntiles, gx, [&](uint32_t t, uint32_t) { atomicAdd(tc + t, 1u); });
     uint32_t big = __ballot_sync(0xffffffffu, ntiles > kOwnTiles);
     while (big) {
         const int src = __ffs(big) - 1;
@@ -135,8 +170,11 @@ __device__ __forceinline__ void count_tiles(uint32_t* tc, int gx, uint2 rc, uint
                                    __shfl_sync(0xffffffffu, rc.y, src));
         const uint32_t bx0 = r.x & 0xFFFFu, by0 = r.x >> 16, bw = (r.y & 0xFFFFu) - bx0;
         const uint32_t bn = bw * ((r.y >> 16) - by0);
-        for (uint32_t i = lane_id(); i < bn; i += 32)
-            atomicAdd(tc + (by0 + i / bw) * (uint32_t)gx + bx0 + i % bw, 1u);
+        const RectRows rr(bw, bn);
+        for (uint32_t i = lane_id(); i < bn; i += 32) {
+            const uint32_t row = rr.row(i);
+            atomicAdd(tc + (by0 + row) * (uint32_t)gx + bx0 + (i - row * bw), 1u);
+        }
     }
 }
 
@@ -156,13 +194,15 @@ __device__ __forceinline__ void bin_rect_range(uint32_t* tc, int gx, uint2 r, ui
                                                uint32_t cap, uint32_t* __restrict__ pair_key,
                                                uint32_t* __restrict__ pair_gauss) {
     const uint32_t bx0 = r.x & 0xFFFFu, by0 = r.x >> 16, bw = (r.y & 0xFFFFu) - bx0;
+    const RectRows rr(bw, hi);
     for (uint32_t i0 = lo; i0 < hi; i0 += 32 * kFly) {
         uint32_t tt[kFly], sl[kFly];
 #pragma unroll
         for (uint32_t j = 0; j < kFly; ++j) {
             const uint32_t i = i0 + j * 32 + lane_id();
             if (i < hi) {
-                tt[j] = (by0 + i / bw) * (uint32_t)gx + bx0 + i % bw;
+                const uint32_t row = rr.row(i);
+                tt[j] = (by0 + row) * (uint32_t)gx + bx0 + (i - row * bw);
                 sl[j] = atomicAdd(tc + tt[j], 1u);
             }
         }
@@ -247,18 +287,10 @@ __device__ __forceinline__ void bin_tiles(uint32_t* tc, int gx, uint2 rc, uint32
     if (own && lane == leader) base = atomicAdd(tc + t0, (uint32_t)__popc(peers));
     if (own) {
         uint32_t tt[kOwnTiles], sl[kOwnTiles];
-        uint32_t kx = 0, t = t0;                    // walks the rectangle row by row
-#pragma unroll
-        for (uint32_t i = 1; i < kOwnTiles; ++i) {
-            if (++kx == w) {
-                kx = 0;
-                t += (uint32_t)gx - w + 1;
-            } else {
-                ++t;
-            }
+        for_own_tiles(t0, w, ntiles, gx, [&](uint32_t t, uint32_t i) {
             tt[i] = t;
-            if (i < ntiles) sl[i] = atomicAdd(tc + t, 1u);
-        }
+            sl[i] = atomicAdd(tc + t, 1u);
+        });
 #pragma unroll
         for (uint32_t i = 1; i < kOwnTiles; ++i)
             if (i < ntiles) put(tt[i], sl[i]);
