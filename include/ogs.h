@@ -331,13 +331,17 @@ ogs_status ogs_blend_fwd(const ogs_rec2d* rec, const uint32_t* pair_gauss,
  * T_final (no per-pair storage); a = min(0.99, o G) has zero derivative where clamped.
  *   rec, pair_gauss, tile_range, T_final, n_last: as produced by the forward
  *   bg: host float[3];  dimg f32[3][H][W] = dL/dimage
- *   drec f32[G][9] (ACCUMULATED, caller zeroes): dL/d(u, v, conic a, conic b, conic c,
- *   opacity, r, g, b) per Gaussian.  Atomic accumulation: float summation order varies.
+ *   drec f32[G][9] (ACCUMULATED, caller zeroes, e.g. with ogs_clear_records): dL/d(u, v, conic
+ *   a, conic b, conic c, opacity, r, g, b) per Gaussian.  Atomic accumulation: float summation
+ *   order varies.
+ * ogs_clear_records — zeroes the rows of the frame's counts->n_gaussians Gaussians (at most
+ *   g_cap) and leaves the rest of a buffer sized for the largest view alone.
  * ------------------------------------------------------------------------------------- */
 ogs_status ogs_blend_bwd(const ogs_rec2d* rec, const uint32_t* pair_gauss,
                          const uint32_t* tile_range, int32_t width, int32_t height,
                          const float* bg /* host float[3] */, const float* T_final,
                          const uint32_t* n_last, const float* dimg, float* drec, void* stream);
+ogs_status ogs_clear_records(float* drec, int64_t g_cap, const ogs_counts* counts, void* stream);
 
 /* ---------------------------------------------------------------------------------------
  * ogs_project_bwd — backward of the EWA projection of ogs_project_bin (Sec. 3.1, Eq. 1):

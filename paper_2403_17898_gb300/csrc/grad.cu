@@ -813,9 +813,16 @@ extern "C" ogs_status ogs_loss_l1(const float* img, const float* target, int64_t
 }
 
 // Adam over the rows whose stamp equals `value` (the anchors a training step selected).  A
-// warp takes 32 rows at a time: their stamps are read in one coalesced load, and the warp then
-// walks the touched ones, its lanes covering a row's elements (rows of up to 64 values in two
-// rounds, longer rows in more); gradients of updated rows are cleared.
+// warp takes kAdamRows rows at a time: their stamps are read in coalesced loads, and the elements of
+// the touched rows form one run that the lanes walk together, kAdamFly elements of a lane in flight
+// (short rows share a warp's round, and no row waits for the one before); gradients of updated rows
+// are cleared.  28 B per element of a touched row, but few rows are touched, so the kernel waits on
+// the round trips stamp -> elements: the more rows a warp looks at together, the fewer of them.  2M
+// anchors, four 1080p views' rows, row lengths 32, 30 and 3: 26, 33 and 12 us; a row at a time took 33, 38 and
+// 29 us, 32 stamps at a time 30, 35 and 24 us.
+constexpr int kAdamRows = 128;
+constexpr int kAdamFly = 4;
+
 __global__ void __launch_bounds__(256) adam_rows_kernel(float* __restrict__ p,
                                                         float* __restrict__ grad,
                                                         float* __restrict__ m,
@@ -825,27 +832,76 @@ __global__ void __launch_bounds__(256) adam_rows_kernel(float* __restrict__ p,
                                                         uint32_t value, float lr, float b1,
                                                         float b2, float eps, float ibc1,
                                                         float ibc2, int zero_grad) {
-    const int lane = (int)lane_id();
+    __shared__ uint8_t s_row[256 / 32][kAdamRows];         // touched rows of the warp, in order
+    const int lane = (int)lane_id(), w = threadIdx.x >> 5;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t r0 = warp * 32; r0 < rows; r0 += nwarps * 32) {
-        const int64_t r = r0 + lane;
-        const bool hit = r < rows && stamp[r] == value;
-        uint32_t todo = __ballot_sync(0xffffffffu, hit);
-        while (todo) {
-            const int b = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const int64_t base = (r0 + b) * (int64_t)row_len;
-            for (int e = lane; e < row_len; e += 32) {
-                float P = p[base + e], G = grad[base + e], M = m[base + e], V = v[base + e];
-                adam_one(P, G, M, V, lr, b1, b2, eps, ibc1, ibc2, zero_grad);
-                p[base + e] = P;
-                m[base + e] = M;
-                v[base + e] = V;
-                if (zero_grad) grad[base + e] = G;
+    for (int64_t r0 = warp * kAdamRows; r0 < rows; r0 += nwarps * kAdamRows) {
+        bool hit[kAdamRows / 32];
+#pragma unroll
+        for (int q = 0; q < kAdamRows / 32; ++q) {
+            const int64_t r = r0 + 32 * q + lane;
+            hit[q] = r < rows && stamp[r] == value;
+        }
+        int n = 0;
+#pragma unroll
+        for (int q = 0; q < kAdamRows / 32; ++q) {
+            const uint32_t todo = __ballot_sync(0xffffffffu, hit[q]);
+            if (hit[q]) s_row[w][n + __popc(todo & lanemask_lt())] = (uint8_t)(32 * q + lane);
+            n += __popc(todo);
+        }
+        if (!n) continue;
+        __syncwarp();
+        const int64_t total = (int64_t)n * row_len;
+        const bool small = total <= 0x7FFFFFFF;            // 32-bit division
+        for (int64_t i0 = lane; i0 < total; i0 += 32 * kAdamFly) {
+            int64_t at[kAdamFly];
+            float P[kAdamFly], G[kAdamFly], M[kAdamFly], V[kAdamFly];
+#pragma unroll
+            for (int u = 0; u < kAdamFly; ++u) {
+                const int64_t i = i0 + 32 * u;
+                if (i < total) {
+                    const uint32_t k = small ? (uint32_t)i / (uint32_t)row_len
+                                             : (uint32_t)((uint64_t)i / (uint32_t)row_len);
+                    at[u] = (r0 + s_row[w][k]) * row_len + (i - (int64_t)k * row_len);
+                    P[u] = p[at[u]]; G[u] = grad[at[u]]; M[u] = m[at[u]]; V[u] = v[at[u]];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kAdamFly; ++u) {
+                if (i0 + 32 * u < total) {
+                    adam_one(P[u], G[u], M[u], V[u], lr, b1, b2, eps, ibc1, ibc2, zero_grad);
+                    p[at[u]] = P[u];
+                    m[at[u]] = M[u];
+                    v[at[u]] = V[u];
+                    if (zero_grad) grad[at[u]] = G[u];
+                }
             }
         }
+        __syncwarp();                                      // the list is rewritten
     }
+}
+
+// The first 9 counts->n_gaussians values of drec to zero (at most 9 g_cap).
+__global__ void __launch_bounds__(256) clear_records_kernel(float* __restrict__ drec, int64_t g_cap,
+                                                            const ogs_counts* __restrict__ counts,
+                                                            int vec) {
+    const int64_t g = counts->n_gaussians, n = 9 * (g < g_cap ? g : g_cap);
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t n4 = vec ? n / 4 : 0;
+    for (int64_t i = i0; i < n4; i += stride)
+        reinterpret_cast<float4*>(drec)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int64_t i = 4 * n4 + i0; i < n; i += stride) drec[i] = 0.f;
+}
+
+extern "C" ogs_status ogs_clear_records(float* drec, int64_t g_cap, const ogs_counts* counts,
+                                        void* stream) {
+    if (!drec || !counts || g_cap < 0) return OGS_ERR_ARG;
+    if (g_cap == 0) return OGS_OK;
+    clear_records_kernel<<<stride_grid(9 * g_cap / 4 + 1, 256, 8), 256, 0, (cudaStream_t)stream>>>(
+        drec, g_cap, counts, aligned(drec, 16));
+    return launch_status();
 }
 
 // stamp[sel_idx[r]] = value for the r < counts->n_selected selected anchors
@@ -876,7 +932,7 @@ extern "C" ogs_status ogs_adam_rows(float* param, float* grad, float* m, float* 
     if (rows == 0) return OGS_OK;
     const double bc1 = 1.0 - pow((double)beta1, (double)step);
     const double bc2 = 1.0 - pow((double)beta2, (double)step);
-    adam_rows_kernel<<<stride_grid((rows + 31) / 32 * 32, 256, 8), 256, 0,
+    adam_rows_kernel<<<stride_grid((rows + kAdamRows - 1) / kAdamRows * 32, 256, 8), 256, 0,
                        (cudaStream_t)stream>>>(param, grad, m, v, rows, row_len, stamp, value,
                                                lr, beta1, beta2, eps, (float)(1.0 / bc1),
                                                (float)(1.0 / bc2), zero_grad);

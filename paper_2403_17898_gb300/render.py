@@ -277,8 +277,7 @@ class Renderer:
         st = stream if stream is not None else torch.cuda.current_stream()
 
         def bb():
-            with torch.cuda.stream(st):
-                self.drec.zero_()
+            abi.clear_records(self.drec, self.counts_t, st)
             abi.blend_bwd(self.rec, self.pair_gauss, self.tile_range, self.W, self.H, bg, self.T,
                           self.n_last, dimg, self.drec, st)
         _stage(timers, "blend_bwd", st, bb)
