@@ -256,13 +256,14 @@ constexpr int kBinTile = kBinThreads * kBinItems;
 constexpr int kWarpSort = 512;           // lists up to this length: one warp, keys in registers
 constexpr int kWarpTiles = 4;            // warps of a warp-sort CTA, one tile at a time each
 constexpr int kWarpGrid = 8 * 152;       // warp-sort CTAs: 8 resident per SM
-constexpr int kSmallSort = 2048;         // longer lists up to this length: 16 KB of keys ..
+constexpr int kSmallSort = 2048;         // longer lists up to this length: merged in 34 KB ..
 constexpr int kSmallGrid = 2 * 152;      // .. in CTAs of kLargeThreads looping over those lists
 constexpr int kLargeThreads = 512;
-constexpr int kLargeSort = 16384;        // longer lists: 128 KB of keys in dynamic shared memory
+constexpr int kLargeMerge = 8192;        // longer lists: merged in 136 KB up to this length, ..
+constexpr int kLargeSort = 16384;        // .. up to this one the network on 128 KB of keys
 constexpr int kLargeGrid = 152;          // CTAs looping over the long lists
-constexpr int kBinsListSort = 4096;      // ogs_sort_bins: lists past kWarpSort, 32 KB of keys ..
-constexpr int kBinsListGrid = 4 * 152;   // .. in CTAs of kLargeThreads, four per SM
+constexpr int kBinsListSort = 4096;      // ogs_sort_bins: lists past kWarpSort, merged in 68 KB ..
+constexpr int kBinsListGrid = 2 * 152;   // .. in CTAs of kLargeThreads, two per SM
 
 __device__ __forceinline__ void rect_of(uint2 r, uint32_t& x0, uint32_t& y0, uint32_t& x1,
                                         uint32_t& y1) {
@@ -781,11 +782,12 @@ static_assert((1 << kPosBits) == kWarpSort, "position field");
 
 // Exact form for a list of 2 <= cnt <= kWarpSort entries: the 512-slot network on the 64-bit
 // keys (depth << 32 | id), read from and written back to the list in place (every read lands
-// in registers before the first write).  Called by a whole warp; kept out of line, since it is
-// the rare path and its code would otherwise crowd the instruction cache.
+// in registers before the first write), or the sorted keys written to `sorted` if that is given.
+// Called by a whole warp; kept out of line, since it is the rare path and its code would
+// otherwise crowd the instruction cache.
 __device__ __noinline__ void warp_sort_exact(const uint32_t* __restrict__ keys,
                                              uint32_t* __restrict__ ids, uint32_t cnt,
-                                             uint32_t lane) {
+                                             uint32_t lane, unsigned long long* sorted) {
     constexpr int kPer = kWarpSort / 32;
     unsigned long long w[kPer];
 #pragma unroll
@@ -798,7 +800,10 @@ __device__ __noinline__ void warp_sort_exact(const uint32_t* __restrict__ keys,
 #pragma unroll
     for (int j = 0; j < kPer; ++j) {
         const uint32_t e = lane * kPer + j;
-        if (e < cnt) ids[e] = (uint32_t)w[j];
+        if (e < cnt) {
+            if (sorted) sorted[e] = w[j];
+            else ids[e] = (uint32_t)w[j];
+        }
     }
 }
 
@@ -870,11 +875,13 @@ __device__ __forceinline__ bool oe_round(uint32_t (&v)[kPer], uint32_t lane, uin
 // id) until a round moves nothing (every neighbour then in order: the list is sorted; runs are
 // short, so one or two rounds usually do); after kFixRounds rounds the list is sorted again
 // from scratch on the exact keys (warp_sort_exact).  Padding slots hold ~0,
-// at or above every real key.
-template <int kPer>
+// at or above every real key.  The sorted ids go back to the list, or with kKeys the sorted
+// exact keys to `sorted` (the list is then a chunk of a longer one).
+template <int kPer, bool kKeys = false>
 __device__ __forceinline__ void warp_sort_list(uint32_t* sd, uint32_t* si, uint2 r, uint32_t lane,
                                                const uint32_t* __restrict__ keys,
-                                               uint32_t* __restrict__ ids) {
+                                               uint32_t* __restrict__ ids,
+                                               unsigned long long* sorted = nullptr) {
     const uint32_t cnt = r.y - r.x;
     uint32_t dmin = 0xFFFFFFFFu, dmax = 0;
 #pragma unroll
@@ -918,9 +925,18 @@ __device__ __forceinline__ void warp_sort_list(uint32_t* sd, uint32_t* si, uint2
             }
         }
         if (!settled) {                     // uniform over the warp
-            warp_sort_exact(keys + r.x, ids + r.x, cnt, lane);
+            warp_sort_exact(keys + r.x, ids + r.x, cnt, lane, kKeys ? sorted : nullptr);
             return;
         }
+    }
+    if constexpr (kKeys) {
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const uint32_t e = v[j] & ((1u << kPosBits) - 1), slot = lane * kPer + j;
+            if (slot < cnt)
+                sorted[slot] = ((unsigned long long)sd[e + e / kPer] << 32) | si[e + e / kPer];
+        }
+        return;
     }
     // slots < cnt hold real keys, whose positions are < cnt: their ids, lane-major, to sd
     __syncwarp();
@@ -965,15 +981,94 @@ __global__ void __launch_bounds__(32 * kWarpTiles, 8) tile_sort_warp(const uint2
     }
 }
 
+// ---------------------------------------------------------------------------------------
+// Lists longer than a warp sorts: the warps of a CTA sort chunks of kWarpSort entries in
+// registers, then the sorted runs are merged pairwise in shared memory, every thread producing
+// an equal stretch of the output from where its diagonal crosses the merge path (a binary search
+// over the two runs; keys are unique).  Latency-bound: a handful of barriers and serial merges of
+// up to 16 keys.  (The bitonic network on 64-bit keys in shared memory, which still serves lists
+// beyond the merge buffers, took 35 barriers and 28 full exchanges for 4500 entries: the 64 long
+// lists of a 128 x 128 view took 16 + 53 us and take 12 + 28 us, those of a 1080p view 20 and 17.)
+// ---------------------------------------------------------------------------------------
+constexpr int kChunkWords = kWarpSort + kWarpSort / 16;    // a chunk's sd / si
+// bytes of the two key buffers for lists of up to n entries (a multiple of kWarpSort): n keys,
+// and n keys or the chunks' sd and si
+constexpr size_t merge_bytes(int n) {
+    return sizeof(unsigned long long) * (size_t)n +
+           2 * sizeof(uint32_t) * kChunkWords * (size_t)(n / kWarpSort);
+}
+
+// shared memory of the longest lists' CTAs
+constexpr size_t kListedSmem = merge_bytes(kLargeMerge);
+static_assert(kListedSmem >= sizeof(unsigned long long) * kLargeSort, "the network's keys fit");
+static_assert(kLargeMerge <= kWarpSort * kLargeThreads / 32, "a chunk per warp");
+
+// One merge level: sorted runs of len keys of src (the last one shorter; cnt keys in all) pairwise
+// into dst; per = output keys per thread, a power of two that divides len.
+__device__ __forceinline__ void merge_level(const unsigned long long* __restrict__ src,
+                                            unsigned long long* __restrict__ dst, uint32_t cnt,
+                                            uint32_t len, uint32_t per) {
+    const uint32_t o = threadIdx.x * per;
+    if (o >= cnt) return;
+    const uint32_t a0 = o & ~(2 * len - 1);
+    const uint32_t a1 = min(a0 + len, cnt), b1 = min(a0 + 2 * len, cnt);
+    const unsigned long long* A = src + a0;
+    const unsigned long long* B = src + a1;
+    const uint32_t na = a1 - a0, nb = b1 - a1, d = o - a0;
+    uint32_t lo = d > nb ? d - nb : 0, hi = min(d, na);
+    while (lo < hi) {                                      // keys of A among the first d outputs
+        const uint32_t mid = (lo + hi) >> 1;
+        if (A[mid] < B[d - 1 - mid]) lo = mid + 1;
+        else hi = mid;
+    }
+    uint32_t i = lo, j = d - lo;
+    const uint32_t end = min(per, na + nb - d);
+    unsigned long long ka = i < na ? A[i] : ~0ull, kb = j < nb ? B[j] : ~0ull;
+    for (uint32_t k = 0; k < end; ++k) {
+        const bool take = ka < kb;
+        dst[o + k] = take ? ka : kb;
+        if (take) ka = ++i < na ? A[i] : ~0ull;
+        else kb = ++j < nb ? B[j] : ~0ull;
+    }
+}
+
+// Sorts the list r of kWarpSort < cnt <= cap entries (cap a multiple of kWarpSort, at most
+// kWarpSort per warp of the CTA); buf holds merge_bytes(cap).
+__device__ __forceinline__ void sort_by_merging(unsigned long long* buf, uint32_t cap, uint2 r,
+                                                const uint32_t* __restrict__ keys,
+                                                uint32_t* __restrict__ ids) {
+    const uint32_t cnt = r.y - r.x, warp = threadIdx.x >> 5;
+    unsigned long long *src = buf, *dst = buf + cap;
+    if (warp * kWarpSort < cnt) {
+        const uint32_t c0 = r.x + warp * kWarpSort;
+        uint32_t* sd = reinterpret_cast<uint32_t*>(dst) + 2 * kChunkWords * warp;
+        warp_sort_list<kWarpSort / 32, true>(sd, sd + kChunkWords,
+                                             make_uint2(c0, min(c0 + (uint32_t)kWarpSort, r.y)),
+                                             lane_id(), keys, ids, src + warp * kWarpSort);
+    }
+    __syncthreads();
+    uint32_t m = 2 * kWarpSort;
+    while (m < cnt) m <<= 1;
+    const uint32_t per = max(m / blockDim.x, 1u);
+    for (uint32_t len = kWarpSort; len < cnt; len <<= 1) {
+        merge_level(src, dst, cnt, len, per);
+        __syncthreads();
+        unsigned long long* t = src;
+        src = dst;
+        dst = t;
+    }
+    for (uint32_t i = threadIdx.x; i < cnt; i += blockDim.x) ids[r.x + i] = (uint32_t)src[i];
+}
+
 // gridDim.x CTAs loop over the tiles listed per scan chunk (chunk c: list[c * kScanChunk ..
-// + nlist[c]]), in chunk order, each list sorted in shared memory (cap keys) or, beyond that,
-// on global memory
+// + nlist[c]]), in chunk order, each list sorted in shared memory (by merging up to merge_cap
+// keys, by the bitonic network up to cap) or, beyond that, on global memory
 template <int kT>
-__global__ void __launch_bounds__(kT) tile_sort_listed(const uint2* __restrict__ range,
+__global__ void __launch_bounds__(kT, 2) tile_sort_listed(const uint2* __restrict__ range,
                                                        const uint32_t* __restrict__ list,
                                                        const uint32_t* __restrict__ nlist,
-                                                       int nchunks, uint32_t cap,
-                                                       const ogs_counts* counts,
+                                                       int nchunks, uint32_t merge_cap,
+                                                       uint32_t cap, const ogs_counts* counts,
                                                        uint32_t* __restrict__ keys,
                                                        uint32_t* __restrict__ ids) {
     pdl_wait();
@@ -987,7 +1082,9 @@ __global__ void __launch_bounds__(kT) tile_sort_listed(const uint2* __restrict__
         while (i >= nlist[c]) i -= nlist[c++];
         const uint2 r = range[list[c * kScanChunk + i]];
         const uint32_t cnt = r.y - r.x;
-        if (cnt <= cap) {
+        if (cnt <= merge_cap) {
+            sort_by_merging(s_k, merge_cap, r, keys, ids);
+        } else if (cnt <= cap) {
             sort_in_smem(s_k, r, keys, ids);
         } else {
             // longer than shared memory holds: the same network on global memory
@@ -1131,15 +1228,15 @@ extern "C" ogs_status ogs_sort_bins(const uint32_t* depth_key, const uint32_t* r
     launch_pdl(tile_sort_warp, dim3(wgrid), dim3(32 * kWarpTiles), 0, st, range, n_tiles, counts,
                (const uint32_t*)bins->pair_key, bins->pair_gauss);
     // every longer list in one launch: up to kBinsListSort keys in shared memory, the rare
-    // longer list by the same network on global memory
-    const size_t smem = sizeof(unsigned long long) * kBinsListSort;
+    // longer list by the network on global memory
     if (cudaFuncSetAttribute(tile_sort_listed<kLargeThreads>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(unsigned long long) * kLargeSort)) != cudaSuccess)
+                             (int)kListedSmem) != cudaSuccess)
         return OGS_ERR_CUDA;
-    launch_pdl(tile_sort_listed<kLargeThreads>, dim3(kBinsListGrid), dim3(kLargeThreads), smem,
-               st, range, s.longl, s.nlong, nchunks, (uint32_t)kBinsListSort, counts,
-               bins->pair_key, bins->pair_gauss);
+    launch_pdl(tile_sort_listed<kLargeThreads>, dim3(kBinsListGrid), dim3(kLargeThreads),
+               merge_bytes(kBinsListSort), st, range, s.longl, s.nlong, nchunks,
+               (uint32_t)kBinsListSort, (uint32_t)kBinsListSort, counts, bins->pair_key,
+               bins->pair_gauss);
     return launch_status();
 }
 
@@ -1181,15 +1278,16 @@ extern "C" ogs_status ogs_sort(const uint32_t* depth_key, const uint32_t* rect, 
     const int wgrid = std::min((n_tiles + kWarpTiles - 1) / kWarpTiles, kWarpGrid);
     launch_pdl(tile_sort_warp, dim3(wgrid), dim3(32 * kWarpTiles), 0, st, range, n_tiles, counts,
                (const uint32_t*)s.keys, pair_gauss);
-    launch_pdl(tile_sort_listed<kLargeThreads>, dim3(kSmallGrid), dim3(kLargeThreads),
-               sizeof(unsigned long long) * kSmallSort, st, range, s.mid, s.nmid, nchunks,
-               (uint32_t)kSmallSort, counts, s.keys, pair_gauss);
-    const size_t smem = sizeof(unsigned long long) * kLargeSort;
     if (cudaFuncSetAttribute(tile_sort_listed<kLargeThreads>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kListedSmem) != cudaSuccess)
         return OGS_ERR_CUDA;
-    launch_pdl(tile_sort_listed<kLargeThreads>, dim3(kLargeGrid), dim3(kLargeThreads), smem, st,
-               range, s.big, s.nbig, nchunks, (uint32_t)kLargeSort, counts, s.keys, pair_gauss);
+    launch_pdl(tile_sort_listed<kLargeThreads>, dim3(kSmallGrid), dim3(kLargeThreads),
+               merge_bytes(kSmallSort), st, range, s.mid, s.nmid, nchunks, (uint32_t)kSmallSort,
+               (uint32_t)kSmallSort, counts, s.keys, pair_gauss);
+    launch_pdl(tile_sort_listed<kLargeThreads>, dim3(kLargeGrid), dim3(kLargeThreads), kListedSmem,
+               st, range, s.big, s.nbig, nchunks, (uint32_t)kLargeMerge, (uint32_t)kLargeSort,
+               counts, s.keys, pair_gauss);
     return launch_status();
 }
 
