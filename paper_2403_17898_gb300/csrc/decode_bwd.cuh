@@ -8,7 +8,6 @@
 namespace ogs {
 namespace db {
 
-constexpr int kDbThreads = 128;
 constexpr int kF = 32;
 constexpr int kH = 32;
 constexpr int kDin = kF + 4;
@@ -125,29 +124,6 @@ __device__ __forceinline__ void dy_cov(const GaussGrad& g, const float (&lvv)[3]
     const float dot = qn[0] * gqa[0] + qn[1] * gqa[1] + qn[2] * gqa[2] + qn[3] * gqa[3];
 #pragma unroll
     for (int e = 0; e < 4; ++e) dy[3 + e] = (gqa[e] - qn[e] * dot) * inv;
-}
-
-// The gradients of decoder m's outputs for Gaussian i of anchor j (row g = r k + i of the
-// Gaussian arrays); with the covariance decoder also the position terms of l_v (dlv) and of the
-// offsets (accumulated in doffs).
-__device__ __forceinline__ void gaussian_dy(const DbArgs& a, int m, size_t g, uint32_t j, int i,
-                                            float w, const float (&lvv)[3], const float* y,
-                                            float* dy, float (&dlv)[3]) {
-    const GaussGrad gg = load_gauss_grad(a, g);
-    if (m == 0) {
-        dy_opacity(gg, w, y, dy);
-    } else if (m == 1) {
-        dy_color(gg, y, dy);
-    } else {
-        dy_cov(gg, lvv, y, dy, dlv);
-        // positions: mu = x_v + O * l_v
-        const float* O = a.offs + ((size_t)j * kK + i) * 3;
-#pragma unroll
-        for (int e = 0; e < 3; ++e) {
-            a.doffs[((size_t)j * kK + i) * 3 + e] += gg.mean[e] * lvv[e];
-            dlv[e] += gg.mean[e] * O[e];
-        }
-    }
 }
 
 constexpr int kDbBlocks = 2 * kSmCount;

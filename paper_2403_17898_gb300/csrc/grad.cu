@@ -159,228 +159,372 @@ __global__ void __launch_bounds__(kPbThreads) project_bwd_kernel(PbArgs a) {
 // decoder backward
 // ---------------------------------------------------------------------------------------
 
-// Row pass: two threads per selected anchor recompute its decoders (weights in shared memory,
-// broadcast reads) and chain the per-Gaussian gradients into dy (110), the hidden
-// pre-activation gradients dp (96) and the feature gradient (dfeat, doffs, dlv accumulate;
-// each anchor appears once per view, so no atomics).  The CTA's first two warps take the
-// opacity and colour decoders of 64 anchors, the last two the covariance decoder (and the
-// position terms) of the same anchors: equal work, no divergence inside a warp; the two
-// feature-gradient halves meet in shared memory.  dy, h, dp and z are written as rows for
-// the weight pass.  Layer 1 runs in outer-product form over a streamed input (only the 32
-// hidden accumulators live in registers), so a thread keeps h, dh and dz (96 values).
-constexpr int kRowAnchors = kDbThreads / 2;
+// Row pass: 64 anchors at a time, the decoders recomputed and differentiated by small matrix products
+// with both operands in shared memory and register blocks of outputs (as the FP32 decoder's):
+//   hidden    a thread owns 4 anchors x 12 hidden units
+//   outputs   4 anchors x the 11 outputs of one Gaussian slot; the thread turns them into that
+//             Gaussian's dy (its gradients were loaded during the product) and its shares of doffs
+//             and dlv
+//   dh        4 anchors x 8 covariance or 16 opacity / colour hidden units, masked by the ReLU into dp
+//   dfeat     4 anchors x 4 features
+// The rows z, h, dy, dp go to scratch for the weight pass.  Each anchor appears once per view, so
+// nothing needs atomics.  Products are packed over anchor pairs and summed in input order.  Bound by
+// the FP32 pipes, shared-memory loads and the gathers' latency: 31k anchors 81 us, against 125 us with
+// two threads per anchor (every weight read once per four products, strided gradient loads).
+constexpr int kRowAnchors = 64;
+constexpr int kRowGroups = kRowAnchors / 4;              // of four anchors
+constexpr int kRowThreads = kRowGroups * kK;             // (anchor group, Gaussian slot)
+constexpr int kRowHid = 12;                              // hidden units per thread
+constexpr int kW2Pitch = kH + 4;                         // conflict-free by slots, 16-byte rows
+static_assert(kRowThreads == 160 && kRowGroups * 8 == 128, "thread roles");
+
+struct __align__(16) RowSmem {
+    float w1[kDin + kMaxApp][3 * kH];    // transposed; rows kDin .. are the appearance weights
+    float w1f[3 * kH][kF];               // W1 restricted to the features
+    float w2[kNOut][kW2Pitch];           // stacked second layers
+    float b1[3 * kH];
+    float b2[kNOut + 2];
+    float h[3 * kH][kRowAnchors];        // hidden activations, then dp
+    float d[kNOut + 3 * kK][kRowAnchors];    // inputs z, then dy and the shares of dlv
+    float rows[kRowAnchors][8];          // anchor index, weight, l_v
+};
+static_assert(kDin + kMaxApp <= kNOut, "z fits under dy");
+static_assert(sizeof(RowSmem) <= 112 * 1024, "two CTAs per SM");
+
+// dh of kN hidden units from h0 (decoder rows row0 .. row0 + nrows of W2 and dy) for anchor group
+// ag, through the ReLU; dp replaces h and goes to the rows.
+template <int kN>
+__device__ __forceinline__ void dh_block(RowSmem& s, const DbArgs& a, int ag, int h0, int row0,
+                                         int nrows, uint32_t base, uint32_t M) {
+    const int hl = h0 % kH;
+    f32x2 acc[kN][2];
+#pragma unroll
+    for (int o = 0; o < kN; ++o) acc[o][0] = acc[o][1] = 0;
+#pragma unroll 2
+    for (int k = 0; k < nrows; ++k) {
+        const float4 d = *reinterpret_cast<const float4*>(&s.d[row0 + k][4 * ag]);
+        const f32x2 d0 = pack2(d.x, d.y), d1 = pack2(d.z, d.w);
+#pragma unroll
+        for (int q = 0; q < kN / 4; ++q) {
+            const float4 w = *reinterpret_cast<const float4*>(&s.w2[row0 + k][hl + 4 * q]);
+            const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const f32x2 w2 = pack2(wv[u], wv[u]);
+                acc[4 * q + u][0] = fma2(w2, d0, acc[4 * q + u][0]);
+                acc[4 * q + u][1] = fma2(w2, d1, acc[4 * q + u][1]);
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kN / 4; ++q) {
+        float dp[4][4];                                  // [hidden][anchor]
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            float* hp = &s.h[h0 + 4 * q + u][4 * ag];
+            const float4 h = *reinterpret_cast<const float4*>(hp);
+            dp[u][0] = h.x > 0.f ? lo2(acc[4 * q + u][0]) : 0.f;
+            dp[u][1] = h.y > 0.f ? hi2(acc[4 * q + u][0]) : 0.f;
+            dp[u][2] = h.z > 0.f ? lo2(acc[4 * q + u][1]) : 0.f;
+            dp[u][3] = h.w > 0.f ? hi2(acc[4 * q + u][1]) : 0.f;
+            *reinterpret_cast<float4*>(hp) = make_float4(dp[u][0], dp[u][1], dp[u][2], dp[u][3]);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+            if (base + 4 * ag + r < M)
+                *reinterpret_cast<float4*>(a.rowP + (size_t)(base + 4 * ag + r) * kRowP + h0 + 4 * q) =
+                    make_float4(dp[0][r], dp[1][r], dp[2][r], dp[3][r]);
+    }
+}
 
 template <bool APP>
-__global__ void __launch_bounds__(kDbThreads, 3) decode_bwd_rows(DbArgs a) {
-    __shared__ __align__(16) float sW1t[3 * kDin * kH];   // [m][i][o]
-    __shared__ __align__(16) float sW1[3 * kH * kDin];    // [m][o][i]
-    __shared__ float sB1[kNB1];
-    __shared__ __align__(16) float sW2[kNOut * kH];
-    __shared__ float sB2[kNOut];
-    __shared__ float sDz[kRowAnchors][kF + 1];
-    __shared__ __align__(16) float sWa[kH * kMaxApp];     // appearance weights [o][c], padded
-    const int napp = a.mlp.A;
-    for (int e = threadIdx.x; e < kH * kMaxApp; e += kDbThreads) {
-        const int o = e / kMaxApp, q = e % kMaxApp;
-        sWa[e] = q < napp ? a.mlp.w1_app[o * napp + q] : 0.f;
-    }
-    for (int e = threadIdx.x; e < 3 * kH * kDin; e += kDbThreads) {
-        const float v = a.mlp.w1[e];
-        sW1[e] = v;
-        const int m = e / (kH * kDin), o = (e / kDin) % kH, i = e % kDin;
-        sW1t[(m * kDin + i) * kH + o] = v;
-    }
-    for (int e = threadIdx.x; e < kNOut * kH; e += kDbThreads)
-        sW2[e] = e < kK * kH ? a.mlp.w2_op[e]
-                             : (e < 4 * kK * kH ? a.mlp.w2_col[e - kK * kH]
-                                                : a.mlp.w2_cov[e - 4 * kK * kH]);
-    for (int e = threadIdx.x; e < kNB1; e += kDbThreads) sB1[e] = a.mlp.b1[e];
-    for (int e = threadIdx.x; e < kNOut; e += kDbThreads)
-        sB2[e] = e < kK ? a.mlp.b2_op[e] : (e < 4 * kK ? a.mlp.b2_col[e - kK] : a.mlp.b2_cov[e - 4 * kK]);
-    __syncthreads();
+__global__ void __launch_bounds__(kRowThreads, 2) decode_bwd_rows(DbArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    RowSmem& s = *reinterpret_cast<RowSmem*>(smem_raw);
     const uint32_t M = a.counts->n_selected;
-    const Cam& c = a.cam;
-    const bool cov_half = threadIdx.x >= kRowAnchors;        // warp-uniform
-    const int slot = threadIdx.x - (cov_half ? kRowAnchors : 0);
-    const int m_lo = cov_half ? 2 : 0, m_hi = cov_half ? 3 : 2;
-    for (uint32_t base = blockIdx.x * kRowAnchors; base < M; base += gridDim.x * kRowAnchors) {
-        const uint32_t r = base + slot;
-        const bool valid = r < M;
-        float dz[kF];
-#pragma unroll
-        for (int i = 0; i < kF; ++i) dz[i] = 0.f;
-        if (valid) {
-        const uint32_t j = a.sel_idx[r];
-        const float w = a.sel_w[r];
-        const float4* f4 = reinterpret_cast<const float4*>(a.feat + (size_t)j * kF);
-        float lvv[3], dlv[3] = {0.f, 0.f, 0.f}, zc[4];
-        float dv[3];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            dv[q] = a.pos[3 * (size_t)j + q] - c.c[q];
-            lvv[q] = a.lv[3 * (size_t)j + q];
+    const uint32_t ntiles = (M + kRowAnchors - 1) / kRowAnchors;
+    if (blockIdx.x >= ntiles) return;
+    const int t = threadIdx.x, napp = a.mlp.A;
+#pragma unroll 8
+    for (int e = t; e < kDin * 3 * kH; e += kRowThreads) {
+        const int i = e / (3 * kH), o = e % (3 * kH);
+        const float v = a.mlp.w1[o * kDin + i];
+        s.w1[i][o] = v;
+        if (i < kF) s.w1f[o][i] = v;
+    }
+    if (APP) {
+        for (int e = t; e < kMaxApp * kH; e += kRowThreads) {
+            const int q = e / kH, o = e % kH;
+            s.w1[kDin + q][kH + o] = q < napp ? a.mlp.w1_app[o * napp + q] : 0.f;
         }
-        const float d = sqrtf(dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2]);
-        zc[0] = dv[0] / d; zc[1] = dv[1] / d; zc[2] = dv[2] / d; zc[3] = d;
-        if (!cov_half) {
+    }
+#pragma unroll 8
+    for (int e = t; e < kNOut * kH; e += kRowThreads)
+        s.w2[e / kH][e % kH] = e < kK * kH ? a.mlp.w2_op[e]
+                                           : (e < 4 * kK * kH ? a.mlp.w2_col[e - kK * kH]
+                                                              : a.mlp.w2_cov[e - 4 * kK * kH]);
+    for (int e = t; e < kNB1; e += kRowThreads) s.b1[e] = a.mlp.b1[e];
+    for (int e = t; e < kNOut; e += kRowThreads)
+        s.b2[e] = e < kK ? a.mlp.b2_op[e] : (e < 4 * kK ? a.mlp.b2_col[e - kK] : a.mlp.b2_cov[e - 4 * kK]);
+    const Cam& c = a.cam;
+    for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const uint32_t base = tile * kRowAnchors;
+        // gather: two threads per anchor, inputs transposed and as rows
+        if (t < 2 * kRowAnchors) {
+            const int al = t % kRowAnchors, half = t / kRowAnchors;
+            const uint32_t r = base + al;
+            const bool valid = r < M;
+            const uint32_t j = valid ? a.sel_idx[r] : 0u;
+            float4 v[4];
+            const float4* f4 = reinterpret_cast<const float4*>(a.feat + (size_t)j * kF) + 4 * half;
             float4* zr = reinterpret_cast<float4*>(a.rowZ + (size_t)r * kRowZ);
 #pragma unroll
-            for (int i = 0; i < kF / 4; ++i) zr[i] = f4[i];
-            zr[kF / 4] = make_float4(zc[0], zc[1], zc[2], zc[3]);
-            zr[kF / 4 + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        float* yrow = a.rowY + (size_t)r * kRowY;
-        if (cov_half) {
+            for (int i = 0; i < 4; ++i) v[i] = valid ? f4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (half == 0) {
+                float dv[3] = {0.f, 0.f, 0.f}, lv[3] = {0.f, 0.f, 0.f}, d = 1.f, w = 0.f;
+                if (valid) {
+                    w = a.sel_w[r];
 #pragma unroll
-            for (int e = 0; e < kRowY; ++e)
-                if (row_out(e) < 0) yrow[e] = 0.f;
-        }
-        const size_t g0 = (size_t)r * kK;
-#pragma unroll 1
-        for (int m = m_lo; m < m_hi; ++m) {
-            float h[kH], dh[kH];
-#pragma unroll
-            for (int o = 0; o < kH; ++o) h[o] = sB1[m * kH + o];
-            // layer 1, outer-product form: h += W1[:, i] z_i over the streamed input
-#pragma unroll 1
-            for (int i4 = 0; i4 < kDin / 4; ++i4) {
-                const float4 zv = i4 < kF / 4 ? f4[i4] : make_float4(zc[0], zc[1], zc[2], zc[3]);
-                const float zz[4] = {zv.x, zv.y, zv.z, zv.w};
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float4* col = reinterpret_cast<const float4*>(sW1t + (m * kDin + 4 * i4 + u) * kH);
-#pragma unroll
-                    for (int q = 0; q < kH / 4; ++q) {
-                        const float4 wv = col[q];
-                        h[4 * q] = fmaf(wv.x, zz[u], h[4 * q]);
-                        h[4 * q + 1] = fmaf(wv.y, zz[u], h[4 * q + 1]);
-                        h[4 * q + 2] = fmaf(wv.z, zz[u], h[4 * q + 2]);
-                        h[4 * q + 3] = fmaf(wv.w, zz[u], h[4 * q + 3]);
+                    for (int q = 0; q < 3; ++q) {
+                        dv[q] = a.pos[3 * (size_t)j + q] - c.c[q];
+                        lv[q] = a.lv[3 * (size_t)j + q];
                     }
+                    d = sqrtf(dv[0] * dv[0] + dv[1] * dv[1] + dv[2] * dv[2]);
+                    zr[kF / 4] = make_float4(dv[0] / d, dv[1] / d, dv[2] / d, d);
+                    zr[kF / 4 + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
                 }
-            }
-            if (APP && m == 1) {           // the colour decoder also sees the code (Sec. 4.4)
-                float code[kMaxApp];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) s.d[kF + q][al] = dv[q] / d;
+                s.d[kF + 3][al] = d;
+                float* rw = s.rows[al];
+                rw[0] = __uint_as_float(j);
+                rw[1] = w;
+                rw[2] = lv[0]; rw[3] = lv[1]; rw[4] = lv[2];
+            } else if (APP) {
 #pragma unroll
                 for (int q = 0; q < kMaxApp; ++q)
-                    code[q] = q < napp ? a.mlp.app[(size_t)j * napp + q] : 0.f;
+                    s.d[kDin + q][al] = valid && q < napp ? a.mlp.app[(size_t)j * napp + q] : 0.f;
+            }
 #pragma unroll
-                for (int o = 0; o < kH; ++o) {
-                    float v = h[o];
+            for (int i = 0; i < 4; ++i) {
+                if (valid) zr[4 * half + i] = v[i];
+                const int k = 16 * half + 4 * i;
+                s.d[k][al] = v[i].x;
+                s.d[k + 1][al] = v[i].y;
+                s.d[k + 2][al] = v[i].z;
+                s.d[k + 3][al] = v[i].w;
+            }
+        }
+        __syncthreads();
+        if (t < 128) {                                   // hidden units
+            const int ag = t % kRowGroups, o0 = t / kRowGroups * kRowHid;
+            f32x2 acc[kRowHid][2];
 #pragma unroll
-                    for (int q = 0; q < kMaxApp; ++q) v = fmaf(sWa[o * kMaxApp + q], code[q], v);
-                    h[o] = v;
+            for (int o = 0; o < kRowHid; ++o) acc[o][0] = acc[o][1] = pack2(s.b1[o0 + o], s.b1[o0 + o]);
+#pragma unroll 4
+            for (int k = 0; k < kDin; ++k) {
+                const float4 z = *reinterpret_cast<const float4*>(&s.d[k][4 * ag]);
+                const f32x2 z0 = pack2(z.x, z.y), z1 = pack2(z.z, z.w);
+#pragma unroll
+                for (int q = 0; q < kRowHid / 4; ++q) {
+                    const float4 w = *reinterpret_cast<const float4*>(&s.w1[k][o0 + 4 * q]);
+                    const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const f32x2 w2 = pack2(wv[u], wv[u]);
+                        acc[4 * q + u][0] = fma2(w2, z0, acc[4 * q + u][0]);
+                        acc[4 * q + u][1] = fma2(w2, z1, acc[4 * q + u][1]);
+                    }
                 }
             }
-            uint32_t mask = 0;
-#pragma unroll
-            for (int o = 0; o < kH; ++o) {
-                mask |= (h[o] > 0.f ? 1u : 0u) << o;
-                h[o] = fmaxf(h[o], 0.f);
-                dh[o] = 0.f;
-            }
-            {
-                float4* hr = reinterpret_cast<float4*>(a.rowH + (size_t)r * kRowH + m * kH);
-#pragma unroll
-                for (int i = 0; i < kH / 4; ++i)
-                    hr[i] = make_float4(h[4 * i], h[4 * i + 1], h[4 * i + 2], h[4 * i + 3]);
-            }
-            const int per = m == 0 ? 1 : (m == 1 ? 3 : 7);
+            if (APP) {                                   // the colour decoder also sees the code
 #pragma unroll 1
-            for (int i = 0; i < kK; ++i) {
-                float y[7], dy[7];
+                for (int k = kDin; k < kDin + kMaxApp; ++k) {
+                    const float4 z = *reinterpret_cast<const float4*>(&s.d[k][4 * ag]);
+                    const f32x2 z0 = pack2(z.x, z.y), z1 = pack2(z.z, z.w);
 #pragma unroll
-                for (int e = 0; e < 7; ++e) {
-                    y[e] = 0.f;
-                    dy[e] = 0.f;
-                    if (e < per) {
-                        const int row = out_base(m) + per * i + e;
-                        const float4* wr = reinterpret_cast<const float4*>(sW2 + row * kH);
-                        float v = sB2[row];
-#pragma unroll
-                        for (int q = 0; q < kH / 4; ++q) {
-                            const float4 wv = wr[q];
-                            v = fmaf(wv.x, h[4 * q], v);
-                            v = fmaf(wv.y, h[4 * q + 1], v);
-                            v = fmaf(wv.z, h[4 * q + 2], v);
-                            v = fmaf(wv.w, h[4 * q + 3], v);
-                        }
-                        y[e] = v;
-                    }
-                }
-                gaussian_dy(a, m, g0 + i, j, i, w, lvv, y, dy, dlv);
-#pragma unroll
-                for (int e = 0; e < 7; ++e) {
-                    if (e < per) {
-                        const int row = out_base(m) + per * i + e;
-                        yrow[out_row(row)] = dy[e];
-                        const float4* wr = reinterpret_cast<const float4*>(sW2 + row * kH);
-#pragma unroll
-                        for (int q = 0; q < kH / 4; ++q) {
-                            const float4 wv = wr[q];
-                            dh[4 * q] = fmaf(wv.x, dy[e], dh[4 * q]);
-                            dh[4 * q + 1] = fmaf(wv.y, dy[e], dh[4 * q + 1]);
-                            dh[4 * q + 2] = fmaf(wv.z, dy[e], dh[4 * q + 2]);
-                            dh[4 * q + 3] = fmaf(wv.w, dy[e], dh[4 * q + 3]);
-                        }
+                    for (int o = 0; o < kRowHid; ++o) {
+                        if (o0 + o < kH || o0 + o >= 2 * kH) continue;
+                        const f32x2 w2 = pack2(s.w1[k][o0 + o], s.w1[k][o0 + o]);
+                        acc[o][0] = fma2(w2, z0, acc[o][0]);
+                        acc[o][1] = fma2(w2, z1, acc[o][1]);
                     }
                 }
             }
-            // through the ReLU, then into the features: dz_i += sum_o W1[o][i] dp_o
 #pragma unroll
-            for (int o = 0; o < kH; ++o) dh[o] = (mask >> o) & 1u ? dh[o] : 0.f;
-            {
-                float4* pr = reinterpret_cast<float4*>(a.rowP + (size_t)r * kRowP + m * kH);
+            for (int q = 0; q < kRowHid / 4; ++q) {
+                float h[4][4];                           // [hidden][anchor]
 #pragma unroll
-                for (int i = 0; i < kH / 4; ++i)
-                    pr[i] = make_float4(dh[4 * i], dh[4 * i + 1], dh[4 * i + 2], dh[4 * i + 3]);
+                for (int u = 0; u < 4; ++u) {
+                    const f32x2* p = acc[4 * q + u];
+                    h[u][0] = fmaxf(lo2(p[0]), 0.f); h[u][1] = fmaxf(hi2(p[0]), 0.f);
+                    h[u][2] = fmaxf(lo2(p[1]), 0.f); h[u][3] = fmaxf(hi2(p[1]), 0.f);
+                    *reinterpret_cast<float4*>(&s.h[o0 + 4 * q + u][4 * ag]) =
+                        make_float4(h[u][0], h[u][1], h[u][2], h[u][3]);
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+                    if (base + 4 * ag + r < M)
+                        *reinterpret_cast<float4*>(a.rowH + (size_t)(base + 4 * ag + r) * kRowH + o0 + 4 * q) =
+                            make_float4(h[0][r], h[1][r], h[2][r], h[3][r]);
             }
-            if (APP && m == 1) {           // code gradient: dapp_c += sum_o Wa[o][c] dp_o
+        }
+        __syncthreads();
+        {                                                // outputs -> dy of one Gaussian slot
+            const int i = t % kK, ag = t / kK;
+            const int row1 = kK + 3 * i, row2 = 4 * kK + 7 * i;
+            GaussGrad gg[4];                             // in flight during the product
+            float O[4][3], dO[4][3];
 #pragma unroll
-                for (int q = 0; q < kMaxApp; ++q) {
-                    if (q < napp) {
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t r = base + 4 * ag + q;
+                if (r < M) {
+                    gg[q] = load_gauss_grad(a, (size_t)r * kK + i);
+                    const size_t o = ((size_t)__float_as_uint(s.rows[4 * ag + q][0]) * kK + i) * 3;
+#pragma unroll
+                    for (int e = 0; e < 3; ++e) {
+                        O[q][e] = a.offs[o + e];
+                        dO[q][e] = a.doffs[o + e];
+                    }
+                }
+            }
+            f32x2 acc[11][2];
+#pragma unroll
+            for (int e = 0; e < 11; ++e) {
+                const float b = s.b2[e == 0 ? i : (e < 4 ? row1 + e - 1 : row2 + e - 4)];
+                acc[e][0] = acc[e][1] = pack2(b, b);
+            }
+#pragma unroll 2
+            for (int o = 0; o < kH; ++o) {
+#pragma unroll
+                for (int m = 0; m < 3; ++m) {
+                    const float4 h = *reinterpret_cast<const float4*>(&s.h[m * kH + o][4 * ag]);
+                    const f32x2 h0 = pack2(h.x, h.y), h1 = pack2(h.z, h.w);
+#pragma unroll
+                    for (int e = m == 0 ? 0 : (m == 1 ? 1 : 4); e < (m == 0 ? 1 : (m == 1 ? 4 : 11)); ++e) {
+                        const float w = s.w2[e == 0 ? i : (e < 4 ? row1 + e - 1 : row2 + e - 4)][o];
+                        acc[e][0] = fma2(pack2(w, w), h0, acc[e][0]);
+                        acc[e][1] = fma2(pack2(w, w), h1, acc[e][1]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int al = 4 * ag + q;
+                const uint32_t r = base + al;
+                float dy[11], dlv[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+                for (int e = 0; e < 11; ++e) dy[e] = 0.f;
+                if (r < M) {
+                    float y[11];
+#pragma unroll
+                    for (int e = 0; e < 11; ++e) y[e] = q & 1 ? hi2(acc[e][q / 2]) : lo2(acc[e][q / 2]);
+                    const float* rw = s.rows[al];
+                    const float lvv[3] = {rw[2], rw[3], rw[4]};
+                    dy_opacity(gg[q], rw[1], y, dy);
+                    dy_color(gg[q], y + 1, dy + 1);
+                    dy_cov(gg[q], lvv, y + 4, dy + 4, dlv);
+                    // positions: mu = x_v + O * l_v
+                    float* dof = a.doffs + ((size_t)__float_as_uint(rw[0]) * kK + i) * 3;
+#pragma unroll
+                    for (int e = 0; e < 3; ++e) {
+                        dof[e] = fmaf(gg[q].mean[e], lvv[e], dO[q][e]);
+                        dlv[e] = fmaf(gg[q].mean[e], O[q][e], dlv[e]);
+                    }
+                    float* yr = a.rowY + (size_t)r * kRowY;
+                    yr[i] = dy[0];
+#pragma unroll
+                    for (int e = 0; e < 3; ++e) yr[kRowCol + 3 * i + e] = dy[1 + e];
+#pragma unroll
+                    for (int e = 0; e < 7; ++e) yr[kRowCov + 7 * i + e] = dy[4 + e];
+                    if (i == 0) {
+#pragma unroll
+                        for (int e = 0; e < kRowY; ++e)
+                            if (row_out(e) < 0) yr[e] = 0.f;
+                    }
+                }
+                s.d[i][al] = dy[0];
+#pragma unroll
+                for (int e = 0; e < 3; ++e) {
+                    s.d[row1 + e][al] = dy[1 + e];
+                    s.d[kNOut + 3 * i + e][al] = dlv[e];
+                }
+#pragma unroll
+                for (int e = 0; e < 7; ++e) s.d[row2 + e][al] = dy[4 + e];
+            }
+        }
+        __syncthreads();
+        // hidden gradients: 64 threads on the covariance decoder, 32 on each other one
+        {
+            const int ag = t % kRowGroups, hg = t / kRowGroups;
+            if (hg < 4) dh_block<8>(s, a, ag, 2 * kH + 8 * hg, 4 * kK, 7 * kK, base, M);
+            else if (hg < 6) dh_block<16>(s, a, ag, kH + 16 * (hg - 4), kK, 3 * kK, base, M);
+            else if (hg < 8) dh_block<16>(s, a, ag, 16 * (hg - 6), 0, kK, base, M);
+            else
+                for (int e = t - 128; e < 3 * kRowAnchors; e += kRowThreads - 128) {
+                    const int al = e % kRowAnchors, q = e / kRowAnchors;     // l_v gradients
+                    if (base + al < M) {
                         float v = 0.f;
 #pragma unroll
-                        for (int o = 0; o < kH; ++o) v = fmaf(sWa[o * kMaxApp + q], dh[o], v);
-                        a.dapp[(size_t)j * napp + q] += v;
+                        for (int i = 0; i < kK; ++i) v += s.d[kNOut + 3 * i + q][al];
+                        a.dlv[3 * (size_t)__float_as_uint(s.rows[al][0]) + q] += v;
+                    }
+                }
+        }
+        __syncthreads();
+        if (t < 128) {                                   // features: opacity and colour, then covariance
+            const int ag = t % kRowGroups, i0 = t / kRowGroups * 4;
+            float4 df[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (base + 4 * ag + q < M)
+                    df[q] = *reinterpret_cast<const float4*>(
+                        a.dfeat + (size_t)__float_as_uint(s.rows[4 * ag + q][0]) * kF + i0);
+            f32x2 acc[2][4][2];
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) acc[m][u][0] = acc[m][u][1] = 0;
+#pragma unroll 4
+                for (int o = m ? 2 * kH : 0; o < (m ? 3 * kH : 2 * kH); ++o) {
+                    const float4 d = *reinterpret_cast<const float4*>(&s.h[o][4 * ag]);
+                    const float4 w = *reinterpret_cast<const float4*>(&s.w1f[o][i0]);
+                    const f32x2 d0 = pack2(d.x, d.y), d1 = pack2(d.z, d.w);
+                    const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        acc[m][u][0] = fma2(pack2(wv[u], wv[u]), d0, acc[m][u][0]);
+                        acc[m][u][1] = fma2(pack2(wv[u], wv[u]), d1, acc[m][u][1]);
                     }
                 }
             }
 #pragma unroll
-            for (int o = 0; o < kH; ++o) {
-                const float4* wr = reinterpret_cast<const float4*>(sW1 + (m * kH + o) * kDin);
+            for (int q = 0; q < 4; ++q) {
+                if (base + 4 * ag + q < M) {
+                    float g[4];
 #pragma unroll
-                for (int i = 0; i < kF / 4; ++i) {
-                    const float4 wv = wr[i];
-                    dz[4 * i] = fmaf(wv.x, dh[o], dz[4 * i]);
-                    dz[4 * i + 1] = fmaf(wv.y, dh[o], dz[4 * i + 1]);
-                    dz[4 * i + 2] = fmaf(wv.z, dh[o], dz[4 * i + 2]);
-                    dz[4 * i + 3] = fmaf(wv.w, dh[o], dz[4 * i + 3]);
+                    for (int u = 0; u < 4; ++u) {
+                        const f32x2 v = add2(acc[0][u][q / 2], acc[1][u][q / 2]);
+                        g[u] = q & 1 ? hi2(v) : lo2(v);
+                    }
+                    *reinterpret_cast<float4*>(
+                        a.dfeat + (size_t)__float_as_uint(s.rows[4 * ag + q][0]) * kF + i0) =
+                        make_float4(df[q].x + g[0], df[q].y + g[1], df[q].z + g[2], df[q].w + g[3]);
                 }
             }
         }
-        if (cov_half) {
+        if (APP) {                                       // code gradient: dapp_c += sum_o Wa[o][c] dp_o
+            for (int e = t; e < kRowAnchors * kMaxApp; e += kRowThreads) {
+                const int al = e % kRowAnchors, q = e / kRowAnchors;
+                if (q < napp && base + al < M) {
+                    float v = 0.f;
 #pragma unroll
-            for (int i = 0; i < kF; ++i) sDz[slot][i] = dz[i];
-#pragma unroll
-            for (int e = 0; e < 3; ++e) a.dlv[3 * (size_t)j + e] += dlv[e];
-        }
-        }
-        __syncthreads();
-        if (valid && !cov_half) {
-            const uint32_t j = a.sel_idx[r];
-            float4* df = reinterpret_cast<float4*>(a.dfeat + (size_t)j * kF);
-#pragma unroll
-            for (int i = 0; i < kF / 4; ++i) {
-                float4 v = df[i];
-                v.x += dz[4 * i] + sDz[slot][4 * i];
-                v.y += dz[4 * i + 1] + sDz[slot][4 * i + 1];
-                v.z += dz[4 * i + 2] + sDz[slot][4 * i + 2];
-                v.w += dz[4 * i + 3] + sDz[slot][4 * i + 3];
-                df[i] = v;
+                    for (int o = 0; o < kH; ++o) v = fmaf(s.w1[kDin + q][kH + o], s.h[kH + o][al], v);
+                    a.dapp[(size_t)__float_as_uint(s.rows[al][0]) * napp + q] += v;
+                }
             }
         }
-        __syncthreads();
+        __syncthreads();                                 // everything is rewritten by the next tile
     }
 }
 
@@ -796,10 +940,12 @@ extern "C" ogs_status ogs_decode_bwd(const float* pos, const float* feat, const 
     DbArgs a{pos, feat, offs, lv, sel_idx, sel_w, counts, *mlp, make_cam(*cam), dmeans, dscales,
              dquats, drec, dfeat, doffs, dlv, sc.rowY, sc.rowH, sc.rowP, sc.rowZ, sc.partial,
              const_cast<float*>(dmlp->app)};
-    if (mlp->A > 0)
-        decode_bwd_rows<true><<<stride_grid(sel_cap, kRowAnchors, 3), kDbThreads, 0, st>>>(a);
-    else
-        decode_bwd_rows<false><<<stride_grid(sel_cap, kRowAnchors, 3), kDbThreads, 0, st>>>(a);
+    const auto rows = mlp->A > 0 ? decode_bwd_rows<true> : decode_bwd_rows<false>;
+    if (cudaFuncSetAttribute(rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(RowSmem)) != cudaSuccess)
+        return OGS_ERR_CUDA;
+    const int64_t tiles = (sel_cap + kRowAnchors - 1) / kRowAnchors;
+    rows<<<(int)(tiles < 2 * kSmCount ? tiles : 2 * kSmCount), kRowThreads, sizeof(RowSmem), st>>>(a);
     if (launch_weight_pass(a, sc, *dmlp, st) != cudaSuccess) return OGS_ERR_CUDA;
     return launch_status();
 }
