@@ -211,15 +211,12 @@ def _stream(stream):
 def camera(cam) -> Camera:
     """synth.Camera (or any object with the same fields) -> ogs_camera."""
     c = Camera()
-    R = np.asarray(cam.R, np.float32).reshape(9)
-    p = np.asarray(cam.campos, np.float32).reshape(3)
-    for i in range(9):
-        c.R[i] = float(R[i])
-    for i in range(3):
-        c.campos[i] = float(p[i])
-    c.fx, c.fy, c.cx, c.cy = (float(np.float32(v)) for v in (cam.fx, cam.fy, cam.cx, cam.cy))
+    c.R[:] = np.asarray(cam.R, np.float32).reshape(9).tolist()
+    c.campos[:] = np.asarray(cam.campos, np.float32).reshape(3).tolist()
+    # the FP32 fields round to nearest on assignment
+    c.fx, c.fy, c.cx, c.cy = float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy)
     c.width, c.height = int(cam.W), int(cam.H)
-    c.znear, c.d_max, c.s = (float(np.float32(v)) for v in (cam.znear, cam.d_max, cam.s))
+    c.znear, c.d_max, c.s = float(cam.znear), float(cam.d_max), float(cam.s)
     return c
 
 
