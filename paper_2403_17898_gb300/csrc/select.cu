@@ -8,8 +8,8 @@
 //                 tile's copy is in flight while the current one is evaluated; the tile's kept
 //                 anchors (index and weight) are written compacted, in ascending order, to the
 //                 tile's slot of a staging area, with the tile's count;
-//   select_emit   one CTA per tile sums the counts of the tiles before it (its output offset)
-//                 and copies its staged entries into place; tile 0 also writes the totals.
+//   select_emit   one CTA per tile (or four) sums the counts of the tiles before it (its output
+//                 offset) and copies the staged entries into place; CTA 0 also writes the totals.
 // No CTA waits on another, so every tile streams at full rate, and only kept anchors (a few
 // percent) are written twice.
 #include <cmath>
@@ -361,12 +361,17 @@ __global__ void __launch_bounds__(kSelThreads, 3) select_eval_gated(
     if ((t >> 5) == 0) tc::tmem_dealloc(tbase, gate::kGTmemCols);
 }
 
-// Pass 2: one CTA per tile.  Its output offset is the sum of the counts of the tiles before
-// it (each CTA reads them itself: at most a few thousand words, from L2); its staged entries
-// are copied to sel_idx / sel_w at that offset, up to the capacity.  Tile 0 also sums every
-// count and writes M, the Gaussian count and the overflow state.
+// Pass 2: one CTA per kEmitTiles tiles.  Its output offset is the sum of the counts of the tiles
+// before it (each CTA reads them itself: at most a few thousand words, from L2); its staged entries
+// are copied to sel_idx / sel_w at that offset, up to the capacity.  CTA 0 also sums every
+// count and writes M, the Gaussian count and the overflow state.  Bound by the latency of the
+// counts: with more tiles than two waves of CTAs (kEmitWave) a CTA takes four, since each wave
+// reads the counts again (8M anchors, 3907 tiles, 3% kept: 8.8 -> 5.6 us; all kept, the whole
+// selection 111 -> 106 us); below that, one, so that a dense selection's copies keep their parallelism.
 constexpr int kEmitThreads = 256;
+constexpr int kEmitWave = 8 * kSmCount;                 // eight CTAs of 256 threads per SM
 
+template <int kEmitTiles>
 __global__ void __launch_bounds__(kEmitThreads) select_emit(const uint32_t* __restrict__ tile_count,
                                                             int nb,
                                                             const uint32_t* __restrict__ st_idx,
@@ -377,11 +382,18 @@ __global__ void __launch_bounds__(kEmitThreads) select_emit(const uint32_t* __re
     pdl_wait();
     pdl_trigger();
     __shared__ unsigned long long s_part[kEmitThreads / 32];
-    const int tile = blockIdx.x;
-    const uint32_t n = tile_count[tile];
+    const int tile = blockIdx.x * kEmitTiles;
+    uint32_t end[kEmitTiles];                     // entries of the tiles up to and with each
+    uint32_t n = 0;
+#pragma unroll
+    for (int q = 0; q < kEmitTiles; ++q) {
+        n += tile + q < nb ? tile_count[tile + q] : 0u;
+        end[q] = n;
+    }
     if (n == 0 && tile != 0) return;
-    const int upto = tile == 0 ? nb : tile;       // tile 0 sums everything (the total)
+    const int upto = tile == 0 ? nb : tile;       // CTA 0 sums everything (the total)
     unsigned long long part = 0;
+#pragma unroll 8
     for (int i = threadIdx.x; i < upto; i += kEmitThreads) part += tile_count[i];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
@@ -399,12 +411,18 @@ __global__ void __launch_bounds__(kEmitThreads) select_emit(const uint32_t* __re
         counts->need_selected = total > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)total;
         if (total > (unsigned long long)cap) atomicOr(&counts->overflow, 1u);
     }
-    const size_t src = (size_t)tile * kSelChunk;
+#pragma unroll 4
     for (uint32_t r = threadIdx.x; r < n; r += kEmitThreads) {
         const unsigned long long p = off + r;
         if (p < (unsigned long long)cap) {
-            sel_idx[p] = st_idx[src + r];
-            sel_w[p] = st_w[src + r];
+            int q = 0;
+            uint32_t before = 0;
+#pragma unroll
+            for (int u = 0; u + 1 < kEmitTiles; ++u)
+                if (r >= end[u]) { q = u + 1; before = end[u]; }
+            const size_t src = (size_t)(tile + q) * kSelChunk + (r - before);
+            sel_idx[p] = st_idx[src];
+            sel_w[p] = st_w[src];
         }
     }
 }
@@ -435,6 +453,17 @@ size_t sel_layout(int64_t N, void* base, SelScratch* s) {
     t.st_w = cv.take<float>(slots);
     if (s) *s = t;
     return cv.off + 256;
+}
+
+void launch_emit(const uint32_t* tile_count, int nb, const uint32_t* st_idx, const float* st_w,
+                 uint32_t* sel_idx, float* sel_w, int64_t cap, int k, ogs_counts* counts,
+                 cudaStream_t st) {
+    if (nb > 2 * kEmitWave)
+        launch_pdl(select_emit<4>, dim3((nb + 3) / 4), dim3(kEmitThreads), 0, st, tile_count, nb,
+                   st_idx, st_w, sel_idx, sel_w, cap, k, counts);
+    else
+        launch_pdl(select_emit<1>, dim3(nb), dim3(kEmitThreads), 0, st, tile_count, nb, st_idx, st_w,
+                   sel_idx, sel_w, cap, k, counts);
 }
 
 // persistent grid of the tile passes: three CTAs per SM, never more than the tiles
@@ -475,9 +504,7 @@ extern "C" ogs_status ogs_lod_select(const float* pos, const uint8_t* level, con
         return OGS_ERR_CUDA;
     launch_pdl(select_tiles, dim3(tile_grid(nb)), dim3(kSelThreads), kStSmem, st, a, sc.st_idx,
                sc.st_w, sc.tile_count, counts, bulk);
-    launch_pdl(select_emit, dim3(nb), dim3(kEmitThreads), 0, st, (const uint32_t*)sc.tile_count,
-               nb, (const uint32_t*)sc.st_idx, (const float*)sc.st_w, sel_idx, sel_w, sel_cap, k,
-               counts);
+    launch_emit(sc.tile_count, nb, sc.st_idx, sc.st_w, sel_idx, sel_w, sel_cap, k, counts, st);
     return launch_status();
 }
 
@@ -530,9 +557,7 @@ extern "C" ogs_status ogs_lod_select_gated(const float* pos, const uint8_t* leve
         return OGS_ERR_CUDA;
     launch_pdl(select_eval_gated, dim3(tile_grid(nb)), dim3(kSelThreads), kSgSmem, st,
                a, feat, img, p_star, sc.st_idx, sc.st_w, sc.tile_count, counts, bulk);
-    launch_pdl(select_emit, dim3(nb), dim3(kEmitThreads), 0, st, (const uint32_t*)sc.tile_count,
-               nb, (const uint32_t*)sc.st_idx, (const float*)sc.st_w, sel_idx, sel_w, sel_cap, k,
-               counts);
+    launch_emit(sc.tile_count, nb, sc.st_idx, sc.st_w, sel_idx, sel_w, sel_cap, k, counts, st);
     return launch_status();
 }
 
