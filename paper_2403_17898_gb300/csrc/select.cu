@@ -365,9 +365,10 @@ __global__ void __launch_bounds__(kSelThreads, 3) select_eval_gated(
 // before it (each CTA reads them itself: at most a few thousand words, from L2); its staged entries
 // are copied to sel_idx / sel_w at that offset, up to the capacity.  CTA 0 also sums every
 // count and writes M, the Gaussian count and the overflow state.  Bound by the latency of the
-// counts: with more tiles than two waves of CTAs (kEmitWave) a CTA takes four, since each wave
+// counts: with more tiles than three waves of CTAs (kEmitWave) a CTA takes four, since each wave
 // reads the counts again (8M anchors, 3907 tiles, 3% kept: 8.8 -> 5.6 us; all kept, the whole
-// selection 111 -> 106 us); below that, one, so that a dense selection's copies keep their parallelism.
+// selection 111 -> 106 us); below that, one, so that a dense selection's copies keep their parallelism
+// (5.2M anchors, all kept: 77 us, with four tiles 80).
 constexpr int kEmitThreads = 256;
 constexpr int kEmitWave = 8 * kSmCount;                 // eight CTAs of 256 threads per SM
 
@@ -458,7 +459,7 @@ size_t sel_layout(int64_t N, void* base, SelScratch* s) {
 void launch_emit(const uint32_t* tile_count, int nb, const uint32_t* st_idx, const float* st_w,
                  uint32_t* sel_idx, float* sel_w, int64_t cap, int k, ogs_counts* counts,
                  cudaStream_t st) {
-    if (nb > 2 * kEmitWave)
+    if (nb > 3 * kEmitWave)
         launch_pdl(select_emit<4>, dim3((nb + 3) / 4), dim3(kEmitThreads), 0, st, tile_count, nb,
                    st_idx, st_w, sel_idx, sel_w, cap, k, counts);
     else

@@ -1,4 +1,4 @@
-"""Selection where its second pass goes from one tile per CTA to four (more than 2432 tiles of 2048
+"""Selection where its second pass goes from one tile per CTA to four (more than 3648 tiles of 2048
 anchors): the entries, their weights and the counts against the selections of two halves of the
 anchors, each of which takes the one-tile form.  Every anchor is judged by itself, so they are equal
 bit for bit."""
@@ -10,7 +10,7 @@ import synth
 
 pytestmark = pytest.mark.gpu
 
-TILE, LINE = 2048, 2432
+TILE, LINE = 2048, 3648
 
 
 def select(abi, torch, pos, level, dL, cam, cap):
