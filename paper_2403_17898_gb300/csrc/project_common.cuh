@@ -178,6 +178,26 @@ __device__ __forceinline__ void count_tiles(uint32_t* tc, int gx, uint2 rc, uint
     }
 }
 
+// Per-tile counts gathered in shared memory first (count_tiles on the CTA's own histogram, then one
+// coalesced atomic per tile that it met), against one scattered atomic per pair in the L2, where the
+// pairs of a crowded tile queue up: the rule for the grids whose histogram fits the plain shared memory of
+// a CTA and for enough Gaussians to pay for clearing and flushing it.  Projection, atomics -> histogram:
+// 41k Gaussians on 64 tiles 24 -> 10 us, 131k on 8160 tiles (28 tiles each) 36 -> 23, 1M of these 173 ->
+// 68, 4200 on 256 tiles 10 -> 10 (the line: 16 per tile).
+constexpr int kHistTiles = 12288;
+constexpr int kHistMinPerTile = 16;
+inline bool use_tile_hist(int64_t n_gauss, int64_t n_tiles) {
+    return n_tiles <= kHistTiles && n_gauss >= kHistMinPerTile * n_tiles;
+}
+// All threads of the CTA call these, with a __syncthreads between them and the counting.
+__device__ __forceinline__ void hist_clear(uint32_t* hist, int n_tiles) {
+    for (int e = threadIdx.x; e < n_tiles; e += blockDim.x) hist[e] = 0u;
+}
+__device__ __forceinline__ void hist_flush(const uint32_t* hist, int n_tiles, uint32_t* tile_count) {
+    for (int e = threadIdx.x; e < n_tiles; e += blockDim.x)
+        if (hist[e] != 0u) atomicAdd(tile_count + e, hist[e]);
+}
+
 // Rectangles of more than kOwnTiles tiles go through the whole warp in chunks of kChunkTiles
 // tiles.  bin_tiles hands each chunk to a list of deferred (Gaussian, chunk) entries that a
 // second pass spreads over the whole grid, so that a warp holding many large near-camera
