@@ -347,10 +347,10 @@ __global__ void __launch_bounds__(kDpThreads, 3) decode_project_tc(DpArgs a) {
     if (w == 0) tc::tmem_dealloc(tbase, kDpTmemCols);
 }
 
-// The per-tile pair counts of the projected rectangles, in a pass of its own where the histogram pays
+// The per-tile pair counts of the projected rectangles, in a pass of its own where the corner table pays
 // (decode_project_tc has no shared memory left for one).  1M Gaussians at 1080p: decode_project_tc 111
-// us with an atomic per pair, 49 without counting, and 33 for this pass, which the shared atomics on
-// crowded tiles bound.
+// us with an atomic per pair, 49 without counting, and 14 for this pass (33 with a shared atomic per
+// pair and whole warps walking large rectangles).
 constexpr int kCountThreads = 1024;
 
 __global__ void __launch_bounds__(kCountThreads, 2) count_rects(const uint2* __restrict__ rect,
@@ -358,24 +358,21 @@ __global__ void __launch_bounds__(kCountThreads, 2) count_rects(const uint2* __r
                                                                 int gy, uint32_t* tile_count) {
     pdl_wait();
     pdl_trigger();
-    extern __shared__ uint32_t hist[];
+    extern __shared__ uint32_t corners[];
     const int64_t n = (int64_t)counts->n_selected * kK;
     if ((int64_t)blockIdx.x * kCountThreads >= n) return;
-    hist_clear(hist, gx * gy);
+    corner_clear(corners, gx, gy);
     __syncthreads();
     for (int64_t base = (int64_t)blockIdx.x * kCountThreads; base < n;
          base += (int64_t)gridDim.x * kCountThreads) {
         const int64_t g = base + threadIdx.x;
-        uint2 rc = g < n ? rect[g] : make_uint2(0, 0);
+        const uint2 rc = g < n ? rect[g] : make_uint2(0, 0);
+        const uint32_t x0 = rc.x & 0xFFFFu, y0 = rc.x >> 16, x1 = rc.y & 0xFFFFu, y1 = rc.y >> 16;
         // after an expired wait the rectangles of a tile were never written: none may leave the grid
-        if ((rc.y & 0xFFFFu) > (uint32_t)gx || (rc.y >> 16) > (uint32_t)gy ||
-            (rc.x & 0xFFFFu) > (rc.y & 0xFFFFu) || (rc.x >> 16) > (rc.y >> 16))
-            rc = make_uint2(0, 0);
-        const uint32_t w = (rc.y & 0xFFFFu) - (rc.x & 0xFFFFu);
-        count_tiles(hist, gx, rc, w * ((rc.y >> 16) - (rc.x >> 16)));
+        if (x0 < x1 && y0 < y1 && x1 <= (uint32_t)gx && y1 <= (uint32_t)gy) corner_add(corners, gx, rc);
     }
     __syncthreads();
-    hist_flush(hist, gx * gy, tile_count);
+    corner_flush(corners, gx, gy, tile_count);
 }
 
 }  // namespace
@@ -418,17 +415,18 @@ extern "C" ogs_status ogs_decode_project_bf16(
     if (cudaFuncSetAttribute(decode_project_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kDpSmem) != cudaSuccess)
         return OGS_ERR_CUDA;
-    const bool hist = tile_count && use_tile_hist(sel_cap * kK, n_tc);
+    const bool corners = tile_count && use_corners(sel_cap * kK, cm.gx, cm.gy);
     DpArgs a{pos, feat, offs, lv, sel_idx, sel_w, counts,
              write_gauss ? *out : ogs_gaussians{nullptr, nullptr, nullptr, nullptr, nullptr},
              write_gauss ? 1 : 0, reinterpret_cast<float4*>(rec), depth_key,
-             reinterpret_cast<uint2*>(rect), tiles, hist ? nullptr : tile_count, img, mlp->app, mlp->A, cm};
+             reinterpret_cast<uint2*>(rect), tiles, corners ? nullptr : tile_count, img, mlp->app, mlp->A, cm};
     const int64_t tiles_cap = (sel_cap + kTM - 1) / kTM;
     const int grid = (int)(tiles_cap < 3 * kSmCount ? tiles_cap : 3 * kSmCount);
     launch_pdl(decode_project_tc, dim3(grid), dim3(kDpThreads), kDpSmem, st, a);
-    if (hist)
+    if (corners)
         launch_pdl(count_rects, dim3(stride_grid(sel_cap * kK, kCountThreads, 2)), dim3(kCountThreads),
-                   sizeof(uint32_t) * n_tc, st, reinterpret_cast<const uint2*>(rect),
+                   sizeof(uint32_t) * corner_entries(cm.gx, cm.gy), st,
+                   reinterpret_cast<const uint2*>(rect),
                    (const ogs_counts*)counts, cm.gx, cm.gy, tile_count);
     return launch_status();
 }

@@ -10,7 +10,7 @@ namespace ogs {
 namespace {
 
 constexpr int kProjThreads = 256;
-constexpr int kHistProjThreads = 512;    // two CTAs per SM: a histogram for half the SM's threads
+constexpr int kCornerThreads = 512;      // counting by corners: two tables per SM
 
 struct ProjArgs {
     ogs_gaussians g;
@@ -25,15 +25,15 @@ struct ProjArgs {
     uint32_t* tile_count;    // optional per-tile pair counts (zeroed before the launch)
 };
 
-template <bool HIST>
-__global__ void __launch_bounds__(HIST ? kHistProjThreads : kProjThreads, HIST ? 2 : 1)
+template <bool CORNERS>
+__global__ void __launch_bounds__(CORNERS ? kCornerThreads : kProjThreads, CORNERS ? 2 : 1)
 project_kernel(ProjArgs a) {
-    extern __shared__ uint32_t hist[];
+    extern __shared__ uint32_t corners[];
     const Cam& c = a.cam;
     const int64_t n = a.count ? (int64_t)*a.count : a.n_fixed;
-    if (HIST) {
+    if (CORNERS) {
         if ((int64_t)blockIdx.x * blockDim.x >= n) return;
-        hist_clear(hist, c.gx * c.gy);
+        corner_clear(corners, c.gx, c.gy);
         __syncthreads();
     }
     // uniform trip count per warp, so the tile counting can use full-warp intrinsics
@@ -61,12 +61,13 @@ project_kernel(ProjArgs a) {
             a.rect[gi] = p.rc;
             a.tiles[gi] = p.ntiles;
         }
-        if (HIST) count_tiles(hist, c.gx, p.rc, p.ntiles);
-        else if (a.tile_count) count_tiles(a.tile_count, c.gx, p.rc, p.ntiles);
+        if (CORNERS) {
+            if (p.ntiles) corner_add(corners, c.gx, p.rc);
+        } else if (a.tile_count) count_tiles(a.tile_count, c.gx, p.rc, p.ntiles);
     }
-    if (HIST) {
+    if (CORNERS) {
         __syncthreads();
-        hist_flush(hist, c.gx * c.gy, a.tile_count);
+        corner_flush(corners, c.gx, c.gy, a.tile_count);
     }
 }
 
@@ -93,9 +94,9 @@ extern "C" ogs_status ogs_project_bin(const ogs_gaussians* g, int64_t n_gauss, i
     ProjArgs a{*g, counts ? &counts->n_gaussians : nullptr, n_gauss, means_relative, cm,
                reinterpret_cast<float4*>(rec), depth_key, reinterpret_cast<uint2*>(rect), tiles,
                tile_count};
-    if (tile_count && use_tile_hist(n_gauss, (int64_t)cm.gx * cm.gy))
-        project_kernel<true><<<stride_grid(n_gauss, kHistProjThreads, 2), kHistProjThreads,
-                               sizeof(uint32_t) * cm.gx * cm.gy, st>>>(a);
+    if (tile_count && use_corners(n_gauss, cm.gx, cm.gy))
+        project_kernel<true><<<stride_grid(n_gauss, kCornerThreads, 2), kCornerThreads,
+                               sizeof(uint32_t) * corner_entries(cm.gx, cm.gy), st>>>(a);
     else
         project_kernel<false><<<stride_grid(n_gauss, kProjThreads, 8), kProjThreads, 0, st>>>(a);
     return launch_status();

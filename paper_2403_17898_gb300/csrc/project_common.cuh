@@ -178,24 +178,66 @@ __device__ __forceinline__ void count_tiles(uint32_t* tc, int gx, uint2 rc, uint
     }
 }
 
-// Per-tile counts gathered in shared memory first (count_tiles on the CTA's own histogram, then one
-// coalesced atomic per tile that it met), against one scattered atomic per pair in the L2, where the
-// pairs of a crowded tile queue up: the rule for the grids whose histogram fits the plain shared memory of
-// a CTA and for enough Gaussians to pay for clearing and flushing it.  Projection, atomics -> histogram:
-// 41k Gaussians on 64 tiles 24 -> 10 us, 131k on 8160 tiles (28 tiles each) 36 -> 23, 1M of these 173 ->
-// 68, 4200 on 256 tiles 10 -> 10 (the line: 16 per tile).
-constexpr int kHistTiles = 12288;
-constexpr int kHistMinPerTile = 16;
-inline bool use_tile_hist(int64_t n_gauss, int64_t n_tiles) {
-    return n_tiles <= kHistTiles && n_gauss >= kHistMinPerTile * n_tiles;
+// Per-tile counts of many Gaussians: a CTA adds each rectangle's four corners (+1, -1, -1, +1) to a
+// (gx + 1) x (gy + 1) table in shared memory and turns the table into counts by sums along the rows and
+// then the columns, one coalesced atomic per tile that it met.  Four shared atomics whatever the
+// rectangle's size, against one scattered atomic per pair in the L2, where the pairs of crowded tiles queue
+// up and large rectangles hold their warp.  The rule: tables within the plain shared memory of a CTA
+// and at most 256 tiles a side (the sums walk a side serially), and enough Gaussians to pay for
+// clearing and summing: 16 per tile, where both took 10 us (4200 Gaussians on 256 tiles).  Projection,
+// an atomic per pair -> corners: 41k Gaussians on 64 tiles 24 -> 10 us; 131k on 8160 tiles, 28 tiles
+// each, 36 -> 20, and 1M of these 172 -> 40; 1M at 1080p with 6 tiles each 57 -> 30.
+constexpr int kCornerEntries = 12288, kCornerSide = 256;
+constexpr int kCornerMinPerTile = 16;
+inline int corner_entries(int gx, int gy) { return (gx + 1) * (gy + 1); }
+inline bool use_corners(int64_t n_gauss, int gx, int gy) {
+    return gx <= kCornerSide && gy <= kCornerSide && corner_entries(gx, gy) <= kCornerEntries &&
+           n_gauss >= (int64_t)kCornerMinPerTile * gx * gy;
 }
-// All threads of the CTA call these, with a __syncthreads between them and the counting.
-__device__ __forceinline__ void hist_clear(uint32_t* hist, int n_tiles) {
-    for (int e = threadIdx.x; e < n_tiles; e += blockDim.x) hist[e] = 0u;
+// All threads of the CTA call corner_clear and corner_flush, with a __syncthreads between them and
+// the additions.
+__device__ __forceinline__ void corner_clear(uint32_t* d, int gx, int gy) {
+    for (int e = threadIdx.x; e < (gx + 1) * (gy + 1); e += blockDim.x) d[e] = 0u;
 }
-__device__ __forceinline__ void hist_flush(const uint32_t* hist, int n_tiles, uint32_t* tile_count) {
-    for (int e = threadIdx.x; e < n_tiles; e += blockDim.x)
-        if (hist[e] != 0u) atomicAdd(tile_count + e, hist[e]);
+__device__ __forceinline__ void corner_add(uint32_t* d, int gx, uint2 rc) {
+    const uint32_t p = (uint32_t)gx + 1;
+    const uint32_t x0 = rc.x & 0xFFFFu, y0 = rc.x >> 16, x1 = rc.y & 0xFFFFu, y1 = rc.y >> 16;
+    atomicAdd(d + y0 * p + x0, 1u);
+    atomicAdd(d + y0 * p + x1, 0xFFFFFFFFu);
+    atomicAdd(d + y1 * p + x0, 0xFFFFFFFFu);
+    atomicAdd(d + y1 * p + x1, 1u);
+}
+__device__ __forceinline__ void corner_flush(uint32_t* d, int gx, int gy, uint32_t* tile_count) {
+    const int p = gx + 1, lane = (int)lane_id();
+    for (int y = threadIdx.x >> 5; y < gy; y += (int)blockDim.x >> 5) {     // a warp per row
+        uint32_t carry = 0;
+        for (int xb = 0; xb < gx; xb += 32) {
+            const int x = xb + lane;
+            uint32_t v = x < gx ? d[y * p + x] : 0u;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t u = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += u;
+            }
+            v += carry;
+            if (x < gx) d[y * p + x] = v;
+            carry = __shfl_sync(0xffffffffu, v, 31);
+        }
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < gx; x += blockDim.x) {                    // a thread per column
+        uint32_t s = 0;
+        for (int yb = 0; yb < gy; yb += 8) {
+            uint32_t v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = yb + i < gy ? d[(yb + i) * p + x] : 0u;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                s += v[i];
+                if (yb + i < gy && s != 0u) atomicAdd(tile_count + (size_t)(yb + i) * gx + x, s);
+            }
+        }
+    }
 }
 
 // Rectangles of more than kOwnTiles tiles go through the whole warp in chunks of kChunkTiles

@@ -1,6 +1,6 @@
-"""Per-tile pair counts where their form changes: a histogram per CTA from 16 Gaussians per tile and up
-to 12288 tiles, counted in the projection or, for the fused decode + projection, in a pass of its own;
-one atomic per pair otherwise.  The counts must be those of the rectangles written beside them."""
+"""Per-tile pair counts where their form changes: a table of corners per CTA from 16 Gaussians per tile,
+up to 12288 entries and 256 tiles a side, filled by the projection or, for the fused decode +
+projection, by a pass of its own; one atomic per pair otherwise.  The counts must be those of the rectangles written beside them."""
 import numpy as np
 import pytest
 
@@ -13,7 +13,10 @@ pytestmark = pytest.mark.gpu
 
 GRIDS = [(48, 32, (1, 95, 96, 511, 512, 513, 3000)),          # 6 tiles
          (1920, 1080, (130_559, 130_560, 400_001)),           # 8160 tiles
-         (2048, 1536, (196_608,)), (2064, 1536, (200_000,))]  # 12288 tiles, 12384
+         (2016, 1520, (194_000,)), (2032, 1520, (194_600,)),   # tables of 127 x 96 = 12192, 128 x 96 = 12288
+         (2048, 1520, (200_000,)),                            # 129 x 96: too large
+         (4096, 64, (17_000,)), (4112, 64, (17_000,)),        # 256 and 257 tiles a side
+         (64, 4096, (17_000,)), (64, 4112, (17_000,))]
 
 
 def counted(rect, gx, gy):
@@ -50,7 +53,7 @@ def test_projection(W, H, n):
 
 
 @pytest.mark.parametrize("W,H,M", [(48, 32, 9), (48, 32, 10), (48, 32, 103), (1920, 1080, 13_055),
-                                   (1920, 1080, 13_056), (1920, 1080, 33_001), (2064, 1536, 20_000)])
+                                   (1920, 1080, 13_056), (1920, 1080, 33_001), (2048, 1520, 20_000)])
 @pytest.mark.parametrize("fill", [1.0, 0.6])     # selected anchors of the capacity
 def test_fused(W, H, M, fill):
     import torch
