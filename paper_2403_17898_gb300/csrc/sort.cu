@@ -251,8 +251,11 @@ bool radix_sort(uint32_t* keys, uint32_t* vals, const uint32_t* n_dev, int64_t n
 // ---------------------------------------------------------------------------------------
 
 constexpr int kBinThreads = 256;
+// rounds of kBinThreads Gaussians per CTA of the packed lists' counting and filling: one where that makes
+// at most one wave of CTAs (each round is a chain of scan, search and atomics: 41k Gaussians, the filling
+// 26 -> 11 us), else four
 constexpr int kBinItems = 4;
-constexpr int kBinTile = kBinThreads * kBinItems;
+constexpr int64_t kBinWave = (int64_t)8 * kSmCount * kBinThreads;
 constexpr int kWarpSort = 512;           // lists up to this length: one warp, keys in registers
 constexpr int kWarpTiles = 4;            // warps of a warp-sort CTA, one tile at a time each
 constexpr int kWarpGrid = 8 * 152;       // warp-sort CTAs: 8 resident per SM
@@ -270,10 +273,10 @@ __device__ __forceinline__ void rect_of(uint2 r, uint32_t& x0, uint32_t& y0, uin
     x0 = r.x & 0xFFFFu; y0 = r.x >> 16; x1 = r.y & 0xFFFFu; y1 = r.y >> 16;
 }
 
-// Block-cooperative walk over the pairs of kBinTile Gaussians (load balanced over pairs, not
+// Block-cooperative walk over the pairs of kItems * kBinThreads Gaussians (load balanced over pairs, not
 // Gaussians): calls f(gaussian, tile) for every pair.  Consecutive pairs of a warp mostly
 // belong to the k Gaussians of one anchor and so often share tiles, which f exploits.
-template <class F>
+template <int kItems, class F>
 __device__ __forceinline__ void for_each_pair(const uint32_t* __restrict__ tiles,
                                               const uint2* __restrict__ rect, uint32_t n,
                                               int gx, F f) {
@@ -281,8 +284,8 @@ __device__ __forceinline__ void for_each_pair(const uint32_t* __restrict__ tiles
     __shared__ uint32_t s_g[kBinThreads];
     __shared__ uint2 s_rect[kBinThreads];
     __shared__ uint32_t ws[kBinThreads / 32];
-    const int64_t base = (int64_t)blockIdx.x * kBinTile;
-    for (int it = 0; it < kBinItems; ++it) {
+    const int64_t base = (int64_t)blockIdx.x * (kItems * kBinThreads);
+    for (int it = 0; it < kItems; ++it) {
         const int64_t i = base + it * kBinThreads + threadIdx.x;
         uint32_t c = 0;
         uint2 rc = make_uint2(0, 0);
@@ -337,13 +340,14 @@ __device__ __forceinline__ uint32_t warp_agg_inc(uint32_t* counter, bool valid, 
     return base + __popc(peers & lanemask_lt());
 }
 
+template <int kItems>
 __global__ void __launch_bounds__(kBinThreads) bin_count(const uint32_t* __restrict__ tiles,
                                                          const uint2* __restrict__ rect,
                                                          const uint32_t* n_dev, int64_t n_cap,
                                                          int gx, uint32_t* __restrict__ tcount) {
     const uint32_t n = count_of(n_dev, n_cap);
-    if ((int64_t)blockIdx.x * kBinTile >= n) return;
-    for_each_pair(tiles, rect, n, gx, [&](bool valid, uint32_t, uint32_t t) {
+    if ((int64_t)blockIdx.x * (kItems * kBinThreads) >= n) return;
+    for_each_pair<kItems>(tiles, rect, n, gx, [&](bool valid, uint32_t, uint32_t t) {
         warp_agg_inc(tcount, valid, t, false);
     });
 }
@@ -572,6 +576,7 @@ __global__ void __launch_bounds__(kScanChunk) bins_scan(const uint32_t* __restri
     }
 }
 
+template <int kItems>
 __global__ void __launch_bounds__(kBinThreads) bin_fill(const uint32_t* __restrict__ tiles,
                                                         const uint2* __restrict__ rect,
                                                         const uint32_t* __restrict__ dkey,
@@ -585,8 +590,8 @@ __global__ void __launch_bounds__(kBinThreads) bin_fill(const uint32_t* __restri
     pdl_trigger();
     if (counts->overflow & 2u) return;
     const uint32_t n = count_of(n_dev, n_cap);
-    if ((int64_t)blockIdx.x * kBinTile >= n) return;
-    for_each_pair(tiles, rect, n, gx, [&](bool valid, uint32_t g, uint32_t t) {
+    if ((int64_t)blockIdx.x * (kItems * kBinThreads) >= n) return;
+    for_each_pair<kItems>(tiles, rect, n, gx, [&](bool valid, uint32_t g, uint32_t t) {
         const uint32_t slot = warp_agg_inc(cursor, valid, t, true);
         if (valid) {
             const uint32_t o = range[t].x + slot;
@@ -1275,16 +1280,20 @@ extern "C" ogs_status ogs_sort(const uint32_t* depth_key, const uint32_t* rect, 
     // the Gaussian count is the device count written by the decoder, or the caller's n_gauss
     const uint32_t* n_dev = n_gauss < 0 ? &counts->n_gaussians : nullptr;
     const int64_t n_cap = n_gauss < 0 ? g_cap : (n_gauss < g_cap ? n_gauss : g_cap);
-    int nb = (int)((n_cap + kBinTile - 1) / kBinTile);
+    const bool one = n_cap <= kBinWave;
+    const int64_t per = (int64_t)kBinThreads * (one ? 1 : kBinItems);
+    int nb = (int)((n_cap + per - 1) / per);
     if (nb < 1) nb = 1;
     const uint2* rc = reinterpret_cast<const uint2*>(rect);
-    if (!tile_count) bin_count<<<nb, kBinThreads, 0, st>>>(tiles, rc, n_dev, n_cap, grid_x, s.tcount);
+    if (!tile_count)
+        (one ? bin_count<1> : bin_count<kBinItems>)<<<nb, kBinThreads, 0, st>>>(tiles, rc, n_dev, n_cap,
+                                                                             grid_x, s.tcount);
     const int nchunks = (n_tiles + kScanChunk - 1) / kScanChunk;
     launch_pdl(tile_scan, dim3(nchunks), dim3(kScanChunk), 0, st,
                tile_count ? tile_count : s.tcount, n_tiles, pair_cap, range, s.cursor, s.mid,
                s.nmid, s.big, s.nbig, counts);
-    launch_pdl(bin_fill, dim3(nb), dim3(kBinThreads), 0, st, tiles, rc, depth_key, n_dev, n_cap,
-               grid_x, range, s.cursor, counts, s.keys, pair_gauss);
+    launch_pdl(one ? bin_fill<1> : bin_fill<kBinItems>, dim3(nb), dim3(kBinThreads), 0, st, tiles, rc,
+               depth_key, n_dev, n_cap, grid_x, range, s.cursor, counts, s.keys, pair_gauss);
     const int wgrid = std::min((n_tiles + kWarpTiles - 1) / kWarpTiles, kWarpGrid);
     launch_pdl(tile_sort_warp, dim3(wgrid), dim3(32 * kWarpTiles), 0, st, range, n_tiles, counts,
                (const uint32_t*)s.keys, pair_gauss);
