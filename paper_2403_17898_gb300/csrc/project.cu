@@ -3,7 +3,8 @@
 //
 // One thread per Gaussian, grid-stride over the device-side count.  HBM-bound: reads 56 B of
 // Gaussian SoA, writes a 48 B record, 4 B depth key, 8 B rect and 4 B tile count; optionally
-// also counts the pairs of every tile (the first step of building the per-tile lists).
+// also counts the pairs of every tile (the first step of building the per-tile lists), by corners or
+// by atomics.  1M Gaussians at 1080p with counts: 30 us, of which the bytes need 18.
 #include "project_common.cuh"
 
 namespace ogs {
