@@ -4,7 +4,7 @@
 //
 // With m1 = G*x, m2 = G*x^2, m3 = G*(x y) and the SSIM map S = A1 A2 / (B1 B2) (A1 = 2 m1 my
 // + C1, A2 = 2 (m3 - m1 my) + C2, B1 = m1^2 + my^2 + C1, B2 = m2 - m1^2 + sy^2 + C2):
-//   dS/dm1 = S (2my/A1 - 2my/A2 - 2m1/B1 + 2m1/B2),  dS/dm2 = -S/B2,  dS/dm3 = 2S/A2,
+//   dS/dm1 = 2 my (A2 - A1)/(B1 B2) + 2 S m1 (1/B2 - 1/B1),  dS/dm2 = -S/B2,  dS/dm3 = 2 A1/(B1 B2),
 // and for the mean SSIM:  d/dx = G*g1 + 2 x (G*g2) + y (G*g3), g_i = dS/dm_i / n.
 // Two passes (moments -> SSIM map and partial maps; blur of the partial maps -> gradient).  A
 // training loop that renders against fixed targets can compute the target's two moments once
@@ -107,11 +107,13 @@ __device__ __forceinline__ void store2(float* p, f32x2 v, bool in1, int vec) {
     }
 }
 __device__ __forceinline__ f32x2 both(float v) { return pack2(v, v); }
-// reciprocals, a few ulp: four of them in place of seven divisions per pixel
+// reciprocals, a few ulp: two of them in place of seven divisions per pixel
 __device__ __forceinline__ f32x2 rcp2(f32x2 v) { return pack2(rcp(lo2(v)), rcp(hi2(v))); }
 
 // The lane's two pixels of the forward pass from their moments: the SSIM values and the partial
-// maps gp_i = dS/dm_i / n.
+// maps gp_i = dS/dm_i / n.  With q = 1 / (B1 B2), S/A1 = A2 q and S/A2 = A1 q, so nothing is divided by
+// A1 or A2: where the covariance passes -C2 / 2, A2 now and then rounds to exactly 0 (about one 1080p
+// image pair in a hundred has such a pixel), and S times its reciprocal would be 0 x inf there.
 __device__ __forceinline__ f32x2 ssim_pixels(f32x2 mx, f32x2 my, f32x2 exx, f32x2 eyy, f32x2 exy,
                                              float inv_n, f32x2& g0, f32x2& g1, f32x2& g2) {
     const f32x2 nx = mul2(mx, both(-1.f)), ny = mul2(my, both(-1.f));
@@ -119,12 +121,12 @@ __device__ __forceinline__ f32x2 ssim_pixels(f32x2 mx, f32x2 my, f32x2 exx, f32x
     const f32x2 A1 = fma2(add2(mx, mx), my, both(kC1)), A2 = add2(add2(vxy, vxy), both(kC2));
     const f32x2 B1 = add2(fma2(mx, mx, mul2(my, my)), both(kC1));
     const f32x2 B2 = add2(add2(vx, vy), both(kC2));
-    const f32x2 iA1 = rcp2(A1), iA2 = rcp2(A2), iB1 = rcp2(B1), iB2 = rcp2(B2);
-    const f32x2 S = mul2(mul2(mul2(A1, A2), iB1), iB2);
-    const f32x2 sS = mul2(S, both(inv_n)), s2 = add2(sS, sS);
-    g0 = mul2(s2, fma2(my, sub2(iA1, iA2), mul2(mx, sub2(iB2, iB1))));
-    g1 = mul2(mul2(sS, both(-1.f)), iB2);
-    g2 = mul2(s2, iA2);
+    const f32x2 iB1 = rcp2(B1), iB2 = rcp2(B2), q = mul2(iB1, iB2);
+    const f32x2 S = mul2(mul2(A1, A2), q);
+    const f32x2 sn = mul2(S, both(inv_n)), qn = mul2(q, both(2.f * inv_n));
+    g0 = fma2(mul2(my, sub2(A2, A1)), qn, mul2(mul2(add2(sn, sn), mx), sub2(iB2, iB1)));
+    g1 = mul2(mul2(sn, both(-1.f)), iB2);
+    g2 = mul2(A1, qn);
     return S;
 }
 
