@@ -11,7 +11,8 @@
 // (ogs_ssim_target_stats) and pass them in, so that the forward pass blurs three moments instead
 // of five.
 //
-// Both passes are the same walk: a warp owns a strip of 64 columns (two per lane) and marches
+// All but large images go by 32 x 32 tiles (ssim_tile below), large ones by column strips: both passes
+// are then the same walk, a warp owns a strip of 64 columns (two per lane) and marches
 // down its rows.  A row pair of the inputs (with a kRad halo; zero outside the image: the
 // zero-padded window) passes through a warp-private shared buffer, is blurred horizontally with
 // its two rows packed in one register pair, and enters the vertical blur at once: ten partial
@@ -19,11 +20,11 @@
 // by one (the shift is the destination of the fused multiply-add), packed over the lane's two
 // columns.  Nothing blurred goes through memory, and no warp waits for another.  Bound by the FP32
 // pipes (66 packed operations per row, two columns and three moments) and the partial maps'
-// traffic.  1080p: forward 57 -> 44 us, backward 54 -> 41 us against 32 x 32 tiles with both blurs
-// staged in shared memory, which spent 250 instructions on a pixel (now 142 and 121); the blurs sum
-// in the same order.  The next row pair is copied asynchronously while the current one is blurred
-// (loads into registers were sunk to their use: 71 and 48 us).  The last strip of the gradient adds
-// the loss, which was a launch of its own.
+// traffic.  1080p: forward 57 -> 44 us, backward 54 -> 41 us against tiles as they then were, which
+// spent 250 instructions on a pixel (strips 142 and 121); the blurs of both forms sum in the same
+// order.  The next row pair is copied asynchronously while the current one is blurred
+// (loads into registers were sunk to their use: 71 and 48 us).  The last strip (or tile) of the
+// gradient adds the loss, which was a launch of its own.
 #include <cmath>
 
 #include "internal.cuh"
@@ -64,7 +65,7 @@ __host__ __device__ constexpr int pass_moments(Pass p) { return p == kMoments5 ?
 // Sums over the image, zeroed by the call.  In 64 bits: a thousand strips add to each.
 struct LossSums {
     double ssim, l1;
-    unsigned int done;      // strips whose gradient is finished
+    unsigned int done;      // strips or tiles whose gradient is finished
 };
 
 struct StripArgs {
@@ -79,7 +80,7 @@ struct StripArgs {
     int H, W, rows;         // rows of a strip
     int64_t n;              // C H W
     float inv_n, lam;
-    unsigned int strips;    // strips of the launch
+    unsigned int parts;     // strips or tiles of the launch
     int vec;                // W even and every plane 8-byte aligned: a lane's columns as one vector
 };
 
@@ -128,6 +129,22 @@ __device__ __forceinline__ f32x2 ssim_pixels(f32x2 mx, f32x2 my, f32x2 exx, f32x
     g1 = mul2(mul2(sn, both(-1.f)), iB2);
     g2 = mul2(A1, qn);
     return S;
+}
+
+// Adds one part's sum of the SSIM map (kMoments) or of |x - y| (kGradient) to the image's.  The last
+// part of the gradient: loss = (1 - lam) * mean |x - y| + lam * (1 - mean SSIM).
+template <Pass kPass>
+__device__ __forceinline__ void add_sum(const StripArgs& a, float local) {
+    atomicAdd(kPass == kGradient ? &a.sums->l1 : &a.sums->ssim, (double)local);
+    if (kPass == kGradient && a.loss) {
+        __threadfence();
+        if (atomicAdd(&a.sums->done, 1u) == a.parts - 1) {
+            __threadfence();
+            const double l1 = *(volatile double*)&a.sums->l1;
+            const double ssim = *(volatile double*)&a.sums->ssim, n = (double)a.n;
+            *a.loss += (float)((1.0 - a.lam) * l1 / n + a.lam * (1.0 - ssim / n));
+        }
+    }
 }
 
 // kMoments: moments -> SSIM map (summed) and the three partial maps.  The five moments are G*x,
@@ -313,39 +330,195 @@ __global__ void __launch_bounds__(32 * kStripWarps, kPass == kMoments5 ? 5 : kCt
     if (kPass != kTargetStats) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) local += __shfl_xor_sync(0xffffffffu, local, o);
-        if (lane == 0) {
-            atomicAdd(kPass == kGradient ? &a.sums->l1 : &a.sums->ssim, (double)local);
-            if (kPass == kGradient && a.loss) {
-                // the last strip: loss = (1 - lam) * mean |x - y| + lam * (1 - mean SSIM)
-                __threadfence();
-                if (atomicAdd(&a.sums->done, 1u) == a.strips - 1) {
-                    __threadfence();
-                    const double l1 = *(volatile double*)&a.sums->l1;
-                    const double ssim = *(volatile double*)&a.sums->ssim, n = (double)a.n;
-                    *a.loss += (float)((1.0 - a.lam) * l1 / n + a.lam * (1.0 - ssim / n));
-                }
-            }
-        }
+        if (lane == 0) add_sum<kPass>(a, local);
     }
 }
 
+// The same passes by tiles, for all but large images: a CTA owns 32 x 32 outputs of one channel, stages
+// them with their halo in shared memory, blurs horizontally into shared memory and vertically into
+// registers (four outputs along the blur per thread from fourteen loaded inputs).  A tile blurs 1.3 rows
+// for each that it keeps, where a strip of ten rows blurs two.  A large image gives strips of more rows,
+// and the tiles' second trip through shared memory loses to them.
+constexpr int kTX = 32, kTY = 32;
+constexpr int kHX = kTX + 2 * kRad, kHY = kTY + 2 * kRad;   // 42 x 42 staged inputs
+constexpr int kTileThreads = 256;
+constexpr int kRun = 4;                                    // outputs of a thread along a blur
+constexpr int kRunSpan = kRun + kWin - 1;                  // their inputs
+static_assert(kTX * (kTY / kRun) == kTileThreads, "a vertical run per thread");
+
+template <Pass kPass>
+__global__ void __launch_bounds__(kTileThreads) ssim_tile(StripArgs a) {
+    constexpr int kIn = pass_inputs(kPass), kM = pass_moments(kPass);
+    static_assert(kPass != kTargetStats, "strips only");
+    __shared__ float s_in[kIn][kHY][kHX + 1];
+    __shared__ float s_h[kM][kHY][kTX + 1];
+    __shared__ float s_red[kTileThreads / 32];
+    pdl_wait();
+    pdl_trigger();
+    const int x0 = blockIdx.x * kTX - kRad, y0 = blockIdx.y * kTY - kRad;
+    const int64_t plane = (int64_t)blockIdx.z * a.H * a.W;
+    {
+        // 6 rows of 42 columns at a time (threads 252 .. 255 idle), every load before any store
+        constexpr int kRowsPer = kTileThreads / kHX, kTimes = (kHY + kRowsPer - 1) / kRowsPer;
+        const int q = threadIdx.x % kHX, r0 = threadIdx.x / kHX, gx = x0 + q;
+        float v[kIn][kTimes];
+#pragma unroll
+        for (int k = 0; k < kTimes; ++k) {
+            const int r = r0 + kRowsPer * k, gy = y0 + r;
+            const bool in = r0 < kRowsPer && r < kHY && gx >= 0 && gx < a.W && gy >= 0 && gy < a.H;
+            const int64_t i = plane + (int64_t)gy * a.W + gx;
+#pragma unroll
+            for (int j = 0; j < kIn; ++j) v[j][k] = in ? a.in[j][i] : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < kTimes; ++k)
+#pragma unroll
+            for (int j = 0; j < kIn; ++j)
+                if (r0 < kRowsPer && r0 + kRowsPer * k < kHY) s_in[j][r0 + kRowsPer * k][q] = v[j][k];
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < kHY * (kTX / kRun); e += kTileThreads) {
+        const int r = e / (kTX / kRun), q0 = e % (kTX / kRun) * kRun;
+        float acc[kM][kRun];
+#pragma unroll
+        for (int j = 0; j < kM; ++j)
+#pragma unroll
+            for (int t = 0; t < kRun; ++t) acc[j][t] = 0.f;
+#pragma unroll
+        for (int k = 0; k < kRunSpan; ++k) {
+            float u[kIn], ch[kM];
+#pragma unroll
+            for (int j = 0; j < kIn; ++j) u[j] = s_in[j][r][q0 + k];
+            if (kPass == kGradient) {
+#pragma unroll
+                for (int j = 0; j < kM; ++j) ch[j] = u[j < kIn ? j : 0];
+            } else {
+                ch[0] = u[0];
+                ch[kPass == kMoments3 ? 1 : 2] = u[0] * u[0];
+                ch[kM - 1] = u[0] * u[1];
+                if (kPass == kMoments5) {
+                    ch[1] = u[1];
+                    ch[kM - 2] = u[1] * u[1];
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < kRun; ++t) {
+                const int tap = k - t;
+                if (tap < 0 || tap >= kWin) continue;
+#pragma unroll
+                for (int j = 0; j < kM; ++j) acc[j][t] = fmaf(a.g.w[tap], ch[j], acc[j][t]);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < kRun; ++t)
+#pragma unroll
+            for (int j = 0; j < kM; ++j) s_h[j][r][q0 + t] = acc[j][t];
+    }
+    __syncthreads();
+    const int qc = threadIdx.x % kTX, r0 = threadIdx.x / kTX * kRun;       // one run per thread
+    const int gx = x0 + kRad + qc, gy = y0 + kRad + r0;
+    const int64_t i0 = plane + (int64_t)gy * a.W + gx;
+    // what the epilogue reads, loaded before the blur: the target's moments, or image and target
+    float ext[2][kRun];
+    if (kPass != kMoments5) {
+        const float* src[2] = {kPass == kGradient ? a.x : a.ystat, kPass == kGradient ? a.y : a.ystat + a.n};
+#pragma unroll
+        for (int t = 0; t < kRun; ++t)
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                ext[j][t] = gx < a.W && gy + t < a.H ? src[j][i0 + (int64_t)t * a.W] : 0.f;
+    }
+    float m[kM][kRun];
+#pragma unroll
+    for (int j = 0; j < kM; ++j)
+#pragma unroll
+        for (int t = 0; t < kRun; ++t) m[j][t] = 0.f;
+#pragma unroll
+    for (int k = 0; k < kRunSpan; ++k) {
+        float h[kM];
+#pragma unroll
+        for (int j = 0; j < kM; ++j) h[j] = s_h[j][r0 + k][qc];
+#pragma unroll
+        for (int t = 0; t < kRun; ++t) {
+            const int tap = k - t;
+            if (tap < 0 || tap >= kWin) continue;
+#pragma unroll
+            for (int j = 0; j < kM; ++j) m[j][t] = fmaf(a.g.w[tap], h[j], m[j][t]);
+        }
+    }
+    float local = 0.f;
+#pragma unroll
+    for (int t = 0; t < kRun; t += 2) {                                    // two rows, packed
+        const bool in0 = gx < a.W && gy + t < a.H, in1 = gx < a.W && gy + t + 1 < a.H;
+        const int64_t i[2] = {i0 + (int64_t)t * a.W, i0 + (int64_t)(t + 1) * a.W};
+        auto pair = [&](int j) { return pack2(m[j][t], m[j][t + 1]); };
+        f32x2 g[3];
+        if (kPass == kGradient) {
+            const f32x2 x = pack2(ext[0][t], ext[0][t + 1]), y = pack2(ext[1][t], ext[1][t + 1]);
+            const f32x2 df = sub2(x, y);
+            const float d0 = lo2(df), d1 = hi2(df);
+            local += (in0 ? fabsf(d0) : 0.f) + (in1 ? fabsf(d1) : 0.f);
+            const f32x2 sgn = pack2(d0 > 0.f ? a.inv_n : (d0 < 0.f ? -a.inv_n : 0.f),
+                                    d1 > 0.f ? a.inv_n : (d1 < 0.f ? -a.inv_n : 0.f));
+            const f32x2 dssim = fma2(y, pair(kM - 1), fma2(add2(x, x), pair(1), pair(0)));
+            g[0] = fma2(both(-a.lam), dssim, mul2(both(1.f - a.lam), sgn));
+        } else {
+            constexpr bool c3 = kPass == kMoments3;
+            const f32x2 S = ssim_pixels(pair(0), c3 ? pack2(ext[0][t], ext[0][t + 1]) : pair(1),
+                                        c3 ? pair(1) : pair(2), c3 ? pack2(ext[1][t], ext[1][t + 1]) : pair(kM - 2),
+                                        pair(kM - 1), a.inv_n, g[0], g[1], g[2]);
+            local += (in0 ? lo2(S) : 0.f) + (in1 ? hi2(S) : 0.f);
+        }
+#pragma unroll
+        for (int j = 0; j < (kPass == kGradient ? 1 : 3); ++j) {
+            if (in0) a.out[j * a.n + i[0]] = lo2(g[j]);
+            if (in1) a.out[j * a.n + i[1]] = hi2(g[j]);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) local += __shfl_xor_sync(0xffffffffu, local, o);
+    if (lane_id() == 0) s_red[threadIdx.x >> 5] = local;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float s = 0.f;
+        for (int k = 0; k < kTileThreads / 32; ++k) s += s_red[k];
+        add_sum<kPass>(a, s);
+    }
+}
+
+// Tiles below this many values C H W, strips from there on (us of a loss call with the target's moments
+// given and without, tiles / strips): 3 x 128 x 128 12.1 / 14.5 and 12.2 / 16.5; 3 x 270 x 480 18.0 / 24.6 and 18.4 /
+// 26.8; 3 x 540 x 960 30.9 / 36.5 and 33.3 / 40.5; 3 x 675 x 1200 45.2 / 47 and 48.9 / 52; 3 x 720 x 1280 49.6 / 48.8 and
+// 51.7 / 54; 3 x 900 x 1600 75.9 / 65.6 and 79.7 / 73.5; 1080p 102 / 88.6 and 109 / 101.
+constexpr int64_t kTileMax = 2600000;
+
 // Rows per strip: as many strips as fit the SMs at once, since the ten halo rows of a strip are
 // blurred twice and a second wave of CTAs would double the time (1080p, 12 strips' warps per SM:
-// 54 rows; 900 CTAs in one wave).  A small image gets strips of as few rows as a pair: its time is
-// one strip's, and twelve rows take less than eighteen (strips of at least eight rows lost 2.5 us of
-// 27 on a 0.2-megapixel image against the tiled form).
+// 54 rows; 900 CTAs in one wave).
 constexpr int kMinRows = 2;
 
+// The target's moments are strips at every size; they take little work a row, so that fewer and longer
+// strips are faster: four CTAs per SM instead of six 480 x 270 6.9 -> 4.8 us, 960 x 540 10.9 -> 8.4, 1080p 27 ->
+// 23.4 (three 27, eight 23.1 but 960 x 540 9.5).
 template <Pass kPass>
 void launch_strips(StripArgs a, int C, cudaStream_t st) {
     const int cols = (a.W + kCols - 1) / kCols;
-    int64_t ny = (int64_t)kSmCount * kCtas / ((int64_t)cols * C);
+    const int ctas = kPass == kTargetStats ? 4 : kCtas;
+    int64_t ny = (int64_t)kSmCount * ctas / ((int64_t)cols * C);
     if (ny < 1) ny = 1;
     const int64_t rows = (a.H + ny * kStripWarps - 1) / (ny * kStripWarps);
     a.rows = (int)(rows < kMinRows ? kMinRows : (rows + 1) / 2 * 2);
     ny = (a.H + (int64_t)a.rows * kStripWarps - 1) / ((int64_t)a.rows * kStripWarps);
-    a.strips = (unsigned)((a.H + a.rows - 1) / a.rows) * (unsigned)cols * (unsigned)C;
+    a.parts = (unsigned)((a.H + a.rows - 1) / a.rows) * (unsigned)cols * (unsigned)C;
     launch_pdl(ssim_strip<kPass>, dim3(cols, (unsigned)ny, C), dim3(32 * kStripWarps), 0, st, a);
+}
+
+template <Pass kPass>
+void launch_pass(StripArgs a, int C, bool tiles, cudaStream_t st) {
+    if (!tiles) return launch_strips<kPass>(a, C, st);
+    const dim3 grid((a.W + kTX - 1) / kTX, (a.H + kTY - 1) / kTY, C);
+    a.parts = grid.x * grid.y * grid.z;
+    launch_pdl(ssim_tile<kPass>, grid, dim3(kTileThreads), 0, st, a);
 }
 
 }  // namespace
@@ -398,13 +571,14 @@ extern "C" ogs_status ogs_loss_l1_ssim(const float* img, const float* target, in
     a.lam = lambda;
     a.vec = W % 2 == 0 && aligned(img, 8) && aligned(target, 8) && aligned(dimg, 8) &&
             aligned(target_stats, 8);
-    if (target_stats) launch_strips<kMoments3>(a, C, st);
-    else launch_strips<kMoments5>(a, C, st);
+    const bool tiles = n < kTileMax && (H + kTY - 1) / kTY <= 65535;       // (the grid's limit)
+    if (target_stats) launch_pass<kMoments3>(a, C, tiles, st);
+    else launch_pass<kMoments5>(a, C, tiles, st);
     for (int j = 0; j < 3; ++j) a.in[j] = gp + j * n;
     a.x = img;
     a.y = target;
     a.out = dimg;
     a.loss = loss;
-    launch_strips<kGradient>(a, C, st);
+    launch_pass<kGradient>(a, C, tiles, st);
     return launch_status();
 }
