@@ -959,16 +959,23 @@ extern "C" ogs_status ogs_loss_l1(const float* img, const float* target, int64_t
 }
 
 // Adam over the rows whose stamp equals `value` (the anchors a training step selected).  A
-// warp takes kAdamRows rows at a time: their stamps are read in coalesced loads, and the elements of
+// warp takes kRows rows at a time: their stamps are read in coalesced loads, and the elements of
 // the touched rows form one run that the lanes walk together, kAdamFly elements of a lane in flight
 // (short rows share a warp's round, and no row waits for the one before); gradients of updated rows
 // are cleared.  28 B per element of a touched row, but few rows are touched, so the kernel waits on
 // the round trips stamp -> elements: the more rows a warp looks at together, the fewer of them.  2M
 // anchors, four 1080p views' rows, row lengths 32, 30 and 3: 26, 33 and 12 us; a row at a time took 33, 38 and
 // 29 us, 32 stamps at a time 30, 35 and 24 us.
-constexpr int kAdamRows = 128;
+// With fewer rows, windows of 128 leave too few warps to share the touched rows: 128 from 48 windows
+// per SM on, 32 (or 64 of short rows) down to kAdamFew rows, four below.  us for windows of 128 / 64 / 32 / 4
+// rows of 32 elements: 1M rows, 6 % touched 16.8 / 16.7 / 16.8 / 30.9; 500k 12.4 / 11.9 / 10.5 / 18.7; 100k, all
+// touched 48.8 / 28.9 / 18.7 / 16.7; 16k, all touched 47.4 / 26.8 / 14.6 / 6.4; 500, all touched 45.3 / 26.9 / 14.5 / 4.4.
+// Rows of 3: 500k, 6 % touched 6.4 / 6.4 / 8.2 / 18.7; 100k, all touched 8.4 / 6.4 / 4.6 / 10.4.
+constexpr int64_t kAdamMany = (int64_t)48 * kSmCount * 128, kAdamFew = 32768;
+constexpr int kAdamShort = 8;            // elements of a short row
 constexpr int kAdamFly = 4;
 
+template <int kRows>
 __global__ void __launch_bounds__(256) adam_rows_kernel(float* __restrict__ p,
                                                         float* __restrict__ grad,
                                                         float* __restrict__ m,
@@ -978,20 +985,21 @@ __global__ void __launch_bounds__(256) adam_rows_kernel(float* __restrict__ p,
                                                         uint32_t value, float lr, float b1,
                                                         float b2, float eps, float ibc1,
                                                         float ibc2, int zero_grad) {
-    __shared__ uint8_t s_row[256 / 32][kAdamRows];         // touched rows of the warp, in order
+    constexpr int kLoads = (kRows + 31) / 32;
+    __shared__ uint8_t s_row[256 / 32][kRows];             // touched rows of the warp, in order
     const int lane = (int)lane_id(), w = threadIdx.x >> 5;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t r0 = warp * kAdamRows; r0 < rows; r0 += nwarps * kAdamRows) {
-        bool hit[kAdamRows / 32];
+    for (int64_t r0 = warp * kRows; r0 < rows; r0 += nwarps * kRows) {
+        bool hit[kLoads];
 #pragma unroll
-        for (int q = 0; q < kAdamRows / 32; ++q) {
+        for (int q = 0; q < kLoads; ++q) {
             const int64_t r = r0 + 32 * q + lane;
-            hit[q] = r < rows && stamp[r] == value;
+            hit[q] = 32 * q + lane < kRows && r < rows && stamp[r] == value;
         }
         int n = 0;
 #pragma unroll
-        for (int q = 0; q < kAdamRows / 32; ++q) {
+        for (int q = 0; q < kLoads; ++q) {
             const uint32_t todo = __ballot_sync(0xffffffffu, hit[q]);
             if (hit[q]) s_row[w][n + __popc(todo & lanemask_lt())] = (uint8_t)(32 * q + lane);
             n += __popc(todo);
@@ -1078,10 +1086,13 @@ extern "C" ogs_status ogs_adam_rows(float* param, float* grad, float* m, float* 
     if (rows == 0) return OGS_OK;
     const double bc1 = 1.0 - pow((double)beta1, (double)step);
     const double bc2 = 1.0 - pow((double)beta2, (double)step);
-    adam_rows_kernel<<<stride_grid((rows + kAdamRows - 1) / kAdamRows * 32, 256, 8), 256, 0,
-                       (cudaStream_t)stream>>>(param, grad, m, v, rows, row_len, stamp, value,
-                                               lr, beta1, beta2, eps, (float)(1.0 / bc1),
-                                               (float)(1.0 / bc2), zero_grad);
+    const int n = rows >= kAdamMany ? 128 : (rows < kAdamFew ? 4 : (row_len <= kAdamShort ? 64 : 32));
+    const auto kernel = n == 128 ? adam_rows_kernel<128>
+                                 : (n == 64 ? adam_rows_kernel<64>
+                                            : (n == 32 ? adam_rows_kernel<32> : adam_rows_kernel<4>));
+    kernel<<<stride_grid((rows + n - 1) / n * 32, 256, 8), 256, 0, (cudaStream_t)stream>>>(
+        param, grad, m, v, rows, row_len, stamp, value, lr, beta1, beta2, eps, (float)(1.0 / bc1),
+        (float)(1.0 / bc2), zero_grad);
     return launch_status();
 }
 
