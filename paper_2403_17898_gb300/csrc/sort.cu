@@ -1002,17 +1002,24 @@ __global__ void __launch_bounds__(32 * kWarpTiles, 32 / kWarpTiles) tile_sort_wa
 // registers, then the sorted runs are merged pairwise in shared memory, every thread producing
 // an equal stretch of the output from where its diagonal crosses the merge path (a binary search
 // over the two runs; keys are unique).  Latency-bound: a handful of barriers and serial merges of
-// up to 16 keys.  (The bitonic network on 64-bit keys in shared memory, which still serves lists
+// up to 16 keys.  Lists of up to 1024 entries take chunks of 128, which eight warps sort, and three
+// merges, instead of two chunks of 512 and one merge: 64 lists of 1000 26.9 -> 24.6 us (the bitonic network
+// 26.4), 8160 of 1000 336 -> 306 (352), 8160 of 600 265 -> 224 (291), the whole building of the lists.  (The bitonic network on 64-bit keys in shared memory, which still serves lists
 // beyond the merge buffers, took 35 barriers and 28 full exchanges for 4500 entries: the 64 long
 // lists of a 128 x 128 view took 16 + 53 us and take 12 + 28 us, those of a 1080p view 20 and 17.)
 // ---------------------------------------------------------------------------------------
-constexpr int kChunkWords = kWarpSort + kWarpSort / 16;    // a chunk's sd / si
+constexpr int kShortChunk = 128;                           // lists of up to kShortMerge entries: chunks ..
+constexpr int kShortMerge = 1024;                          // .. for eight warps instead of two
+__host__ __device__ constexpr int chunk_words(int chunk) { return chunk + 32; }            // a chunk's sd / si
 // bytes of the two key buffers for lists of up to n entries (a multiple of kWarpSort): n keys,
 // and n keys or the chunks' sd and si
 constexpr size_t merge_bytes(int n) {
     return sizeof(unsigned long long) * (size_t)n +
-           2 * sizeof(uint32_t) * kChunkWords * (size_t)(n / kWarpSort);
+           2 * sizeof(uint32_t) * chunk_words(kWarpSort) * (size_t)(n / kWarpSort);
 }
+static_assert(2 * chunk_words(kShortChunk) * (kShortMerge / kShortChunk) * sizeof(uint32_t) +
+                      sizeof(unsigned long long) * kSmallSort <= merge_bytes(kSmallSort),
+              "the short chunks' sd and si fit the smaller buffers");
 
 // shared memory of the longest lists' CTAs
 constexpr size_t kListedSmem = merge_bytes(kLargeMerge);
@@ -1048,25 +1055,35 @@ __device__ __forceinline__ void merge_level(const unsigned long long* __restrict
     }
 }
 
+// The warps of the CTA sort the list's chunks of 32 kPer entries into src; their buffers lie in dst.
+template <int kPer>
+__device__ __forceinline__ void sort_chunks(unsigned long long* src, unsigned long long* dst, uint2 r,
+                                            const uint32_t* __restrict__ keys,
+                                            uint32_t* __restrict__ ids) {
+    constexpr uint32_t kChunk = 32 * kPer, kWords = chunk_words(kChunk);
+    const uint32_t warp = threadIdx.x >> 5, c0 = r.x + warp * kChunk;
+    if (c0 < r.y) {
+        uint32_t* sd = reinterpret_cast<uint32_t*>(dst) + 2 * kWords * warp;
+        warp_sort_list<kPer, true>(sd, sd + kWords, make_uint2(c0, min(c0 + kChunk, r.y)), lane_id(),
+                                   keys, ids, src + warp * kChunk);
+    }
+}
+
 // Sorts the list r of kWarpSort < cnt <= cap entries (cap a multiple of kWarpSort, at most
-// kWarpSort per warp of the CTA); buf holds merge_bytes(cap).
+// kWarpSort per warp of the CTA, at least kSmallSort); buf holds merge_bytes(cap).
 __device__ __forceinline__ void sort_by_merging(unsigned long long* buf, uint32_t cap, uint2 r,
                                                 const uint32_t* __restrict__ keys,
                                                 uint32_t* __restrict__ ids) {
-    const uint32_t cnt = r.y - r.x, warp = threadIdx.x >> 5;
+    const uint32_t cnt = r.y - r.x;
     unsigned long long *src = buf, *dst = buf + cap;
-    if (warp * kWarpSort < cnt) {
-        const uint32_t c0 = r.x + warp * kWarpSort;
-        uint32_t* sd = reinterpret_cast<uint32_t*>(dst) + 2 * kChunkWords * warp;
-        warp_sort_list<kWarpSort / 32, true>(sd, sd + kChunkWords,
-                                             make_uint2(c0, min(c0 + (uint32_t)kWarpSort, r.y)),
-                                             lane_id(), keys, ids, src + warp * kWarpSort);
-    }
+    const uint32_t chunk = cnt <= kShortMerge ? kShortChunk : kWarpSort;
+    if (cnt <= kShortMerge) sort_chunks<kShortChunk / 32>(src, dst, r, keys, ids);
+    else sort_chunks<kWarpSort / 32>(src, dst, r, keys, ids);
     __syncthreads();
     uint32_t m = 2 * kWarpSort;
     while (m < cnt) m <<= 1;
     const uint32_t per = max(m / blockDim.x, 1u);
-    for (uint32_t len = kWarpSort; len < cnt; len <<= 1) {
+    for (uint32_t len = chunk; len < cnt; len <<= 1) {
         merge_level(src, dst, cnt, len, per);
         __syncthreads();
         unsigned long long* t = src;
