@@ -169,6 +169,8 @@ class Renderer:
             G = self.g_cap
             dev = "cuda"
             self.drec = torch.zeros(G, 9, device=dev)
+            # counters of the view whose gradients drec holds (none yet): the rest of it is zero
+            self.drec_counts = torch.zeros_like(self.counts_t)
             self.dmeans = torch.empty(G, 3, device=dev)
             self.dscales = torch.empty(G, 3, device=dev)
             self.dquats = torch.empty(G, 4, device=dev)
@@ -271,13 +273,16 @@ class Renderer:
         as the forward) or ogs_explicit_gaussians_bwd.  Anchor gradients accumulate into
         ``grads`` (feat, offs, lv[, app] or offs, lv, ex.*), decoder gradients into the arrays
         of ``dmlp_struct`` (an abi.mlp_struct).  ``on_drec(st)`` runs after the blend backward
-        (per-Gaussian statistics read self.drec there)."""
+        (per-Gaussian statistics read self.drec there: this view's Gaussians, zero past them)."""
         self._grad_buffers()
         c = abi.camera(cam)
         st = stream if stream is not None else torch.cuda.current_stream()
 
         def bb():
-            abi.clear_records(self.drec, self.counts_t, st)
+            # the rows of the view before; the next backward clears this view's
+            abi.clear_records(self.drec, self.drec_counts, st)
+            with torch.cuda.stream(st):
+                self.drec_counts.copy_(self.counts_t)
             abi.blend_bwd(self.rec, self.pair_gauss, self.tile_range, self.W, self.H, bg, self.T,
                           self.n_last, dimg, self.drec, st)
         _stage(timers, "blend_bwd", st, bb)
