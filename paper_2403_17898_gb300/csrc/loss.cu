@@ -152,11 +152,10 @@ __device__ __forceinline__ void add_sum(const StripArgs& a, float local) {
 // kGradient: blur of the partial maps -> dSSIM/dx = G*gp0 + 2 x (G*gp1) + y (G*gp2);
 // out = (1 - lam) sign(x - y) / n - lam dSSIM/dx, and the L1 sum.
 // kTargetStats: G*y and G*y^2.
-// CTAs per SM that the registers allow (kMoments5: five).  More CTAs at 128 registers recompute what
-// they cannot keep: 8 CTAs 50 and 48 us.
+// CTAs per SM that the registers allow: 144 for kMoments3, 156 for kGradient, 166 for kMoments5.  More CTAs at 128 registers recompute what they cannot keep: 8 CTAs 50 and 48 us.
 constexpr int kCtas = 6;
 template <Pass kPass>
-__global__ void __launch_bounds__(32 * kStripWarps, kPass == kMoments5 ? 5 : kCtas) ssim_strip(StripArgs a) {
+__global__ void __launch_bounds__(32 * kStripWarps, kCtas) ssim_strip(StripArgs a) {
     constexpr int kIn = pass_inputs(kPass), kM = pass_moments(kPass);
     constexpr bool kExtra = kPass == kMoments3 || kPass == kGradient;
     // a row pair of the inputs, the two rows of a column together; what its epilogue reads
