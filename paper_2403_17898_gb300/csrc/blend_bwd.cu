@@ -156,7 +156,8 @@ struct PairState {
 };
 
 // One entry's (s, w) at both pixels and their step towards the front.  A pixel that skipped the
-// entry (!ok) has alpha = 0, which leaves its state as it is.  kCareful: the entry can clamp
+// entry (!ok) has alpha = 0, which leaves its state as it is: the approximate reciprocal of 1 is
+// exactly 1 (its bound of an ulp alone would not say so; the blend tests walk past 600 skipped entries).  kCareful: the entry can clamp
 // alpha (whose gradient is then zero), or something is not finite (0 x inf): the exact selections.
 template <bool kCareful>
 __device__ __forceinline__ float4 pair_step(PairState& p, bool ok0, bool ok1, float q0, float q1,
