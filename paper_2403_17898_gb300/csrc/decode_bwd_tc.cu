@@ -21,7 +21,8 @@
 // Gaussian, consecutive Gaussians on consecutive threads, with all of a thread's loads issued
 // first: 64 anchors at a time, their outputs staged in shared memory, dy in place of y, stored as
 // whole rows by one bulk copy.  (One CTA per SM and one thread per half an anchor, whose loads
-// were strided by ten Gaussians: 100k anchors 248 us; now 145 us.)
+// were strided by ten Gaussians: 100k anchors 248 us; now 145 us.)  128 registers, two CTAs' worth, with 252
+// bytes spilled.
 // Operands live in shared memory in the no-swizzle K-major core-matrix layout; every mbarrier
 // wait is bounded and on expiry the kernel sets ogs_counts.timeout, waits (bounded) for the MMAs
 // in flight, releases TMEM and exits.

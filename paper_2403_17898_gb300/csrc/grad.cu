@@ -3,10 +3,11 @@
 //
 // project_bwd: one thread per Gaussian; recomputes the forward quantities and chains
 //   d(u, v, conic) -> d(mean, scale, unit quaternion).
-// decode_bwd: one thread per selected anchor recomputes its three decoders and produces
-//   d(feature), d(offsets), d(l_v); the weight gradients are block-level products
-//   dY^T H and dPre^T Z of the block's anchors (staged in shared memory), each element owned
-//   by one thread, written as per-block partials and summed by a deterministic reduction.
+// decode_bwd (FP32; decode_bwd_tc.cu has the tensor-core rows): a row pass recomputes the three decoders
+//   of 64 anchors at a time by register-blocked products and produces d(feature), d(offsets), d(l_v)
+//   and the rows z, h, dy, dp; a weight pass forms dY^T H and dP^T Z of the rows (staged in shared
+//   memory), a 4 x 8 block of elements per thread, written as per-block partials and summed by a
+//   deterministic reduction.
 #include "internal.cuh"
 #include "decode_bwd.cuh"
 #include "tc.cuh"
@@ -170,7 +171,8 @@ __global__ void __launch_bounds__(kPbThreads) project_bwd_kernel(PbArgs a) {
 // The rows z, h, dy, dp go to scratch for the weight pass.  Each anchor appears once per view, so
 // nothing needs atomics.  Products are packed over anchor pairs and summed in input order.  Bound by
 // the FP32 pipes, shared-memory loads and the gathers' latency: 31k anchors 81 us, against 125 us with
-// two threads per anchor (every weight read once per four products, strided gradient loads).
+// two threads per anchor (every weight read once per four products, strided gradient loads).  168
+// registers with 144 bytes spilled, two CTAs per SM.
 constexpr int kRowAnchors = 64;
 constexpr int kRowGroups = kRowAnchors / 4;              // of four anchors
 constexpr int kRowThreads = kRowGroups * kK;             // (anchor group, Gaussian slot)

@@ -183,10 +183,14 @@ __device__ __forceinline__ void count_tiles(uint32_t* tc, int gx, uint2 rc, uint
 // then the columns, one coalesced atomic per tile that it met.  Four shared atomics whatever the
 // rectangle's size, against one scattered atomic per pair in the L2, where the pairs of crowded tiles queue
 // up and large rectangles hold their warp.  The rule: tables within the plain shared memory of a CTA
-// and at most 256 tiles a side (the sums walk a side serially), and enough Gaussians to pay for
-// clearing and summing: 16 per tile, where both took 10 us (4200 Gaussians on 256 tiles).  Projection,
-// an atomic per pair -> corners: 41k Gaussians on 64 tiles 24 -> 10 us; 131k on 8160 tiles, 28 tiles
-// each, 36 -> 20, and 1M of these 172 -> 40; 1M at 1080p with 6 tiles each 57 -> 30.
+// and at most 256 tiles a side (the sums walk a side serially), and room for enough Gaussians to pay for
+// clearing and summing: 16 per tile, where both took 10 us (4200 Gaussians on 256 tiles).  The room is
+// the caller's capacity, since the view's count is on the device.  Projection, an atomic per pair ->
+// corners: 41k Gaussians on 64 tiles 24 -> 10 us; 131k on 8160 tiles, 28 tiles each, 36 -> 20, and 1M
+// of these 172 -> 40; 1M at 1080p with 6 tiles each 57 -> 30.  A sparse view in large buffers, kernel alone:
+// 1080p, 500 Gaussians 6.7 -> 8.8 us, 8k 7.5 -> 9.5, 12k 16.5 -> 9.8, 24k 9.7 -> 9.5, 40k 16.5 -> 9.9; 128 x 128, 500
+// 5.1 -> 5.9, 8k 5.7 -> 5.9, 12k 6.6 -> 6.0.  (Taking the atomic route in the kernel below 12k by the view's
+// count gave those back and cost the dense views 4 %: 250k at 1080p 15.6 -> 16.2.)
 constexpr int kCornerEntries = 12288, kCornerSide = 256;
 constexpr int kCornerMinPerTile = 16;
 inline int corner_entries(int gx, int gy) { return (gx + 1) * (gy + 1); }

@@ -2,14 +2,21 @@
 // rectangle covers it, in ascending depth, ties by Gaussian id.
 //
 // Lists are short (hundreds of entries, a few thousand at most), so instead of sorting all
-// (tile, depth) pairs globally the work is split by tile:
-//   1. per-tile pair counts (atomics over each Gaussian's rectangle) and their exclusive scan,
-//      which gives every tile's range directly;
+// (tile, depth) pairs globally the work is split by tile, in one of two forms.
+// Packed lists (ogs_sort):
+//   1. per-tile pair counts (handed in by the projection, which forms them by atomics or by corner
+//      tables, or counted here) and their exclusive scan, which gives every tile's range;
 //   2. block-cooperative fill: each pair is written into its tile's range at an atomic cursor
-//      slot as (depth key, Gaussian id), in arbitrary order;
-//   3. one CTA per tile sorts its range by the 64-bit key (depth bits << 32 | id) with a
-//      bitonic network in shared memory (lists longer than the shared-memory capacity use the
-//      same network on global memory).
+//      slot as (depth key, Gaussian id), in arbitrary order.
+// Regions (ogs_sort_bins): one pass writes each pair into its tile's region of fixed size at the slot
+// that the tile's counter returns; large rectangles are put off and shared out in chunks.
+// Then every list is sorted by the 64-bit key (depth bits << 32 | id):
+//   up to 512 entries     one warp, on 32-bit keys (quantised depth, position) in registers, ties mended
+//                         on the exact keys;
+//   up to 8192 (regions 4096)  a CTA: chunks sorted so by its warps (128 entries for lists of up to 1024,
+//                         else 512), then merged along merge paths in shared memory;
+//   up to 16384 (packed)  a bitonic network in shared memory;
+//   longer                the network on global memory.
 // The key is unique per Gaussian, so the order is fully determined: the same lists as one
 // stable sort of (tile, depth) keys in Gaussian-id order, without multi-pass global traffic.
 //
@@ -252,8 +259,10 @@ bool radix_sort(uint32_t* keys, uint32_t* vals, const uint32_t* n_dev, int64_t n
 
 constexpr int kBinThreads = 256;
 // rounds of kBinThreads Gaussians per CTA of the packed lists' counting and filling: one where that makes
-// at most one wave of CTAs (each round is a chain of scan, search and atomics: 41k Gaussians, the filling
-// 26 -> 11 us), else four
+// at most one wave of CTAs for the capacity (the view's own count is on the device), else four.  Each
+// round is a chain of scan, search and atomics: 41k Gaussians, the filling 26 -> 11 us; ogs_sort with
+// counts given, 1080p, 2k Gaussians 28.0 -> 18.0 us, 40k 54.0 -> 49.8, 140k 124 -> 104 (a few views of 160k to
+// 310k with huge rectangles take 2 to 5 % longer)
 constexpr int kBinItems = 4;
 constexpr int64_t kBinWave = (int64_t)8 * kSmCount * kBinThreads;
 constexpr int kWarpSort = 512;           // lists up to this length: one warp, keys in registers
