@@ -11,6 +11,7 @@ import math
 
 import numpy as np
 import torch
+from torch.multiprocessing.reductions import StorageWeakRef
 
 from . import abi
 
@@ -515,7 +516,7 @@ class Trainer(Renderer):
         self.dimg = torch.zeros(3, self.H, self.W, device=dev)
         self.loss = torch.zeros(1, device=dev)
         self.loss_scratch = None
-        self._ssim_stats = {}            # target data_ptr -> (version, window moments)
+        self._ssim_stats = {}    # target data_ptr -> (version, window moments, its storage)
         if self.ssim_lambda > 0:
             self.loss_scratch = torch.empty(abi.loss_l1_ssim_scratch_bytes(3, self.H, self.W),
                                             dtype=torch.uint8, device=dev)
@@ -560,13 +561,15 @@ class Trainer(Renderer):
 
     def _target_stats(self, target, st):
         """The SSIM window moments of a target, computed once per target tensor (recomputed if
-        the tensor was modified in place since)."""
+        the tensor was modified in place since, or freed and its memory taken by another)."""
         key = target.data_ptr()
         hit = self._ssim_stats.get(key)
-        if hit is None or hit[0] != target._version or hit[1].shape[1:] != target.shape:
+        if (hit is None or hit[0] != target._version or hit[1].shape[1:] != target.shape
+                or hit[2].expired()):
             stats = torch.empty((2,) + tuple(target.shape), device="cuda")
             abi.ssim_target_stats(target, stats, st)
-            hit = (target._version, stats)
+            # the storage lives: its addresses are its own
+            hit = (target._version, stats, StorageWeakRef(target.untyped_storage()))
             self._ssim_stats[key] = hit
         return hit[1]
 
