@@ -336,12 +336,18 @@ ogs_status ogs_blend_fwd(const ogs_rec2d* rec, const uint32_t* pair_gauss,
  *   order varies.
  * ogs_clear_records — zeroes the rows of the frame's counts->n_gaussians Gaussians (at most
  *   g_cap) and leaves the rest of a buffer sized for the largest view alone.
+ * ogs_renew_records — prepares a buffer that is zero but for the rows of the frame before for the
+ *   next frame's blend backward: zeroes those rows, so that the whole buffer is zero.  held[0] =
+ *   rows written since the buffer was zeroed (0 for a new one; becomes counts->n_gaussians),
+ *   held[1] = 0; both are kept between calls.
  * ------------------------------------------------------------------------------------- */
 ogs_status ogs_blend_bwd(const ogs_rec2d* rec, const uint32_t* pair_gauss,
                          const uint32_t* tile_range, int32_t width, int32_t height,
                          const float* bg /* host float[3] */, const float* T_final,
                          const uint32_t* n_last, const float* dimg, float* drec, void* stream);
 ogs_status ogs_clear_records(float* drec, int64_t g_cap, const ogs_counts* counts, void* stream);
+ogs_status ogs_renew_records(float* drec, int64_t g_cap, const ogs_counts* counts,
+                             uint32_t* held /* device u32[2] */, void* stream);
 
 /* ---------------------------------------------------------------------------------------
  * ogs_project_bwd — backward of the EWA projection of ogs_project_bin (Sec. 3.1, Eq. 1):

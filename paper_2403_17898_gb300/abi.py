@@ -118,6 +118,7 @@ _SIGS = {
     "ogs_scan_nonfinite": (C.c_int, [_P, _I64, _P, C.c_uint32, _P]),
     "ogs_counts_status": (C.c_int, [_P, C.c_uint32]),
     "ogs_clear_records": (C.c_int, [_P, _I64, _P, _P]),
+    "ogs_renew_records": (C.c_int, [_P, _I64, _P, _P, _P]),
     "ogs_stamp_selected": (C.c_int, [_P, _P, _I64, _P, C.c_uint32, _P]),
     "ogs_adam_rows": (C.c_int, [_P, _P, _P, _P, _I64, _I32, _P, C.c_uint32, C.c_float,
                                 C.c_float, C.c_float, C.c_float, _I32, _I32, _P]),
@@ -390,6 +391,11 @@ def blend_bwd(rec, pair_gauss, tile_range, width, height, bg, T_final, n_last, d
 def clear_records(drec, counts, stream=None):
     _check(lib().ogs_clear_records(_ptr(drec), drec.shape[0], _ptr(counts), _stream(stream)),
            "ogs_clear_records")
+
+
+def renew_records(drec, counts, held, stream=None):
+    _check(lib().ogs_renew_records(_ptr(drec), drec.shape[0], _ptr(counts), _ptr(held),
+                                   _stream(stream)), "ogs_renew_records")
 
 
 def project_bwd(g, n_gauss, means_relative, cam, rect, drec, dmeans, dscales, dquats,

@@ -1038,17 +1038,24 @@ __global__ void __launch_bounds__(256) adam_rows_kernel(float* __restrict__ p,
     }
 }
 
-// The first 9 counts->n_gaussians values of drec to zero (at most 9 g_cap).
+// The first 9 counts->n_gaussians values of drec to zero (at most 9 g_cap); with `held`, the first
+// 9 held[0], and held[0] becomes counts->n_gaussians once every CTA has read it (held[1] counts them).
 __global__ void __launch_bounds__(256) clear_records_kernel(float* __restrict__ drec, int64_t g_cap,
                                                             const ogs_counts* __restrict__ counts,
-                                                            int vec) {
-    const int64_t g = counts->n_gaussians, n = 9 * (g < g_cap ? g : g_cap);
+                                                            uint32_t* held, int vec) {
+    const int64_t g = held ? held[0] : counts->n_gaussians, n = 9 * (g < g_cap ? g : g_cap);
     const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t n4 = vec ? n / 4 : 0;
     for (int64_t i = i0; i < n4; i += stride)
         reinterpret_cast<float4*>(drec)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int64_t i = 4 * n4 + i0; i < n; i += stride) drec[i] = 0.f;
+    if (!held) return;
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(held + 1, 1u) == gridDim.x - 1) {
+        held[0] = counts->n_gaussians;
+        held[1] = 0u;
+    }
 }
 
 extern "C" ogs_status ogs_clear_records(float* drec, int64_t g_cap, const ogs_counts* counts,
@@ -1056,7 +1063,16 @@ extern "C" ogs_status ogs_clear_records(float* drec, int64_t g_cap, const ogs_co
     if (!drec || !counts || g_cap < 0) return OGS_ERR_ARG;
     if (g_cap == 0) return OGS_OK;
     clear_records_kernel<<<stride_grid(9 * g_cap / 4 + 1, 256, 8), 256, 0, (cudaStream_t)stream>>>(
-        drec, g_cap, counts, aligned(drec, 16));
+        drec, g_cap, counts, nullptr, aligned(drec, 16));
+    return launch_status();
+}
+
+extern "C" ogs_status ogs_renew_records(float* drec, int64_t g_cap, const ogs_counts* counts,
+                                        uint32_t* held, void* stream) {
+    if (!drec || !counts || !held || g_cap < 0) return OGS_ERR_ARG;
+    if (g_cap == 0) return OGS_OK;
+    clear_records_kernel<<<stride_grid(9 * g_cap / 4 + 1, 256, 8), 256, 0, (cudaStream_t)stream>>>(
+        drec, g_cap, counts, held, aligned(drec, 16));
     return launch_status();
 }
 

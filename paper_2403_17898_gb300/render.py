@@ -170,8 +170,8 @@ class Renderer:
             G = self.g_cap
             dev = "cuda"
             self.drec = torch.zeros(G, 9, device=dev)
-            # counters of the view whose gradients drec holds (none yet): the rest of it is zero
-            self.drec_counts = torch.zeros_like(self.counts_t)
+            # rows of drec that the last backward wrote (none yet): the rest of it is zero
+            self.drec_held = torch.zeros(2, dtype=torch.int32, device=dev)
             self.dmeans = torch.empty(G, 3, device=dev)
             self.dscales = torch.empty(G, 3, device=dev)
             self.dquats = torch.empty(G, 4, device=dev)
@@ -280,10 +280,7 @@ class Renderer:
         st = stream if stream is not None else torch.cuda.current_stream()
 
         def bb():
-            # the rows of the view before; the next backward clears this view's
-            abi.clear_records(self.drec, self.drec_counts, st)
-            with torch.cuda.stream(st):
-                self.drec_counts.copy_(self.counts_t)
+            abi.renew_records(self.drec, self.counts_t, self.drec_held, st)
             abi.blend_bwd(self.rec, self.pair_gauss, self.tile_range, self.W, self.H, bg, self.T,
                           self.n_last, dimg, self.drec, st)
         _stage(timers, "blend_bwd", st, bb)

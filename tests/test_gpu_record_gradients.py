@@ -30,3 +30,25 @@ def test_rows_past_the_view_are_zero(precision):
     # the same view gives the same gradients whatever came before (float atomics: order of sums)
     for a, b in ((0, 2), (1, 3)):
         assert (seen[a] - seen[b]).norm() <= 1e-4 * seen[a].norm()
+
+
+@pytest.mark.parametrize("cap,off", [(1, 0), (1000, 0), (1000, 1), (200_000, 0)])
+def test_renewed_rows(cap, off):
+    """ogs_renew_records: the rows of the frame before go to zero, nothing else is touched, and the next
+    call clears this frame's."""
+    import torch
+    abi = lib_ready()
+    buf = torch.zeros(cap * 9 + 16, device="cuda")
+    drec = buf[off:off + cap * 9].reshape(cap, 9)
+    counts = torch.zeros(8, dtype=torch.int32, device="cuda")
+    held = torch.zeros(2, dtype=torch.int32, device="cuda")
+    before = 0
+    for n in (cap, cap // 2, 0, 1, cap // 3, cap + 5, cap):
+        counts[1] = n
+        buf.fill_(2.0)
+        abi.renew_records(drec, counts, held)
+        want = torch.full_like(buf, 2.0)
+        want[off:off + 9 * min(before, cap)] = 0
+        assert torch.equal(buf, want)
+        assert held.tolist() == [n, 0]
+        before = n
