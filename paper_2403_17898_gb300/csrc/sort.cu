@@ -807,9 +807,10 @@ static_assert((1 << kPosBits) == kWarpSort, "position field");
 
 // Exact form for a list of 2 <= cnt <= kWarpSort entries: the 512-slot network on the 64-bit
 // keys (depth << 32 | id), read from and written back to the list in place (every read lands
-// in registers before the first write), or the sorted keys written to `sorted` if that is given.
+// in registers before the first write), or with kKeys the sorted keys written to `sorted`.
 // Called by a whole warp; kept out of line, since it is the rare path and its code would
 // otherwise crowd the instruction cache.
+template <bool kKeys>
 __device__ __noinline__ void warp_sort_exact(const uint32_t* __restrict__ keys,
                                              uint32_t* __restrict__ ids, uint32_t cnt,
                                              uint32_t lane, unsigned long long* sorted) {
@@ -826,7 +827,7 @@ __device__ __noinline__ void warp_sort_exact(const uint32_t* __restrict__ keys,
     for (int j = 0; j < kPer; ++j) {
         const uint32_t e = lane * kPer + j;
         if (e < cnt) {
-            if (sorted) sorted[e] = w[j];
+            if (kKeys) sorted[e] = w[j];
             else ids[e] = (uint32_t)w[j];
         }
     }
@@ -950,7 +951,7 @@ __device__ __forceinline__ void warp_sort_list(uint32_t* sd, uint32_t* si, uint2
             }
         }
         if (!settled) {                     // uniform over the warp
-            warp_sort_exact(keys + r.x, ids + r.x, cnt, lane, kKeys ? sorted : nullptr);
+            warp_sort_exact<kKeys>(keys + r.x, ids + r.x, cnt, lane, sorted);
             return;
         }
     }
