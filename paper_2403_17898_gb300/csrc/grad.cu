@@ -968,12 +968,14 @@ extern "C" ogs_status ogs_loss_l1(const float* img, const float* target, int64_t
 // the round trips stamp -> elements: the more rows a warp looks at together, the fewer of them.  2M
 // anchors, four 1080p views' rows, row lengths 32, 30 and 3: 26, 33 and 12 us; a row at a time took 33, 38 and
 // 29 us, 32 stamps at a time 30, 35 and 24 us.
-// With fewer rows, windows of 128 leave too few warps to share the touched rows: 128 from 48 windows
-// per SM on, 32 (or 64 of short rows) down to kAdamFew rows, four below.  us for windows of 128 / 64 / 32 / 4
-// rows of 32 elements: 1M rows, 6 % touched 16.8 / 16.7 / 16.8 / 30.9; 500k 12.4 / 11.9 / 10.5 / 18.7; 100k, all
-// touched 48.8 / 28.9 / 18.7 / 16.7; 16k, all touched 47.4 / 26.8 / 14.6 / 6.4; 500, all touched 45.3 / 26.9 / 14.5 / 4.4.
-// Rows of 3: 500k, 6 % touched 6.4 / 6.4 / 8.2 / 18.7; 100k, all touched 8.4 / 6.4 / 4.6 / 10.4.
-constexpr int64_t kAdamMany = (int64_t)48 * kSmCount * 128, kAdamFew = 32768;
+// With fewer rows, windows of 128 leave too few warps to share the touched rows: 128 from 24 windows
+// per SM on (16 for short rows), 32 (64) down to kAdamFew rows, four below.  us for windows of 128 / 64 / 32 / 4
+// rows of 32 elements: 500k rows, 2 % touched 6.8 / 8.4 / 7.8 / 14.5, 6 % 12.5 / 12.4 / 10.6 / 18.7; 350k, 2 % 6.4 / 7.2 /
+// 6.4 / 12.3, 6 % 10.5 / 10.5 / 9.6 / 14.5; 100k, all touched 48.7 / 28.9 / 18.8 / 16.7; 16k, all touched 47.4 / 26.8 /
+// 14.6 / 6.4; 500, all touched 45.3 / 26.9 / 14.5 / 4.4.  Rows of 3: 350k, 2 % touched 4.4 / 6.4 / 6.3 / 12.5; 100k, all
+// touched 8.4 / 6.4 / 4.4 / 10.4.
+constexpr int64_t kAdamWindow = (int64_t)kSmCount * 128;               // one window of 128 rows per SM
+constexpr int64_t kAdamMany = 24 * kAdamWindow, kAdamManyShort = 16 * kAdamWindow, kAdamFew = 32768;
 constexpr int kAdamShort = 8;            // elements of a short row
 constexpr int kAdamFly = 4;
 
@@ -1039,7 +1041,9 @@ __global__ void __launch_bounds__(256) adam_rows_kernel(float* __restrict__ p,
 }
 
 // The first 9 counts->n_gaussians values of drec to zero (at most 9 g_cap); with `held`, the first
-// 9 held[0], and held[0] becomes counts->n_gaussians once every CTA has read it (held[1] counts them).
+// 9 held[0], and held[0] becomes counts->n_gaussians once every CTA has read it (held[1] counts them; two
+// CTAs per SM, since the atomics queue up: views of up to 600k Gaussians as without held, 4.2 to 6.3 us, with eight 5.1
+// to 6.3; counted before the clearing, beside the others' reads of held[0], eight took 11.5 to 13.9).
 __global__ void __launch_bounds__(256) clear_records_kernel(float* __restrict__ drec, int64_t g_cap,
                                                             const ogs_counts* __restrict__ counts,
                                                             uint32_t* held, int vec) {
@@ -1071,7 +1075,7 @@ extern "C" ogs_status ogs_renew_records(float* drec, int64_t g_cap, const ogs_co
                                         uint32_t* held, void* stream) {
     if (!drec || !counts || !held || g_cap < 0) return OGS_ERR_ARG;
     if (g_cap == 0) return OGS_OK;
-    clear_records_kernel<<<stride_grid(9 * g_cap / 4 + 1, 256, 8), 256, 0, (cudaStream_t)stream>>>(
+    clear_records_kernel<<<stride_grid(9 * g_cap / 4 + 1, 256, 2), 256, 0, (cudaStream_t)stream>>>(
         drec, g_cap, counts, held, aligned(drec, 16));
     return launch_status();
 }
@@ -1104,7 +1108,9 @@ extern "C" ogs_status ogs_adam_rows(float* param, float* grad, float* m, float* 
     if (rows == 0) return OGS_OK;
     const double bc1 = 1.0 - pow((double)beta1, (double)step);
     const double bc2 = 1.0 - pow((double)beta2, (double)step);
-    const int n = rows >= kAdamMany ? 128 : (rows < kAdamFew ? 4 : (row_len <= kAdamShort ? 64 : 32));
+    const bool is_short = row_len <= kAdamShort;
+    const int n = rows >= (is_short ? kAdamManyShort : kAdamMany) ? 128
+                                                                  : (rows < kAdamFew ? 4 : (is_short ? 64 : 32));
     const auto kernel = n == 128 ? adam_rows_kernel<128>
                                  : (n == 64 ? adam_rows_kernel<64>
                                             : (n == 32 ? adam_rows_kernel<32> : adam_rows_kernel<4>));

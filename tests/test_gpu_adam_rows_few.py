@@ -7,13 +7,14 @@ from gpu_helpers import lib_ready
 
 pytestmark = pytest.mark.gpu
 
-FEW, MANY = 32768, 48 * 152 * 128      # rows from which windows of 32 (64) and 128 rows are taken
+FEW, WIN = 32768, 152 * 128      # rows from which windows of 32 (64) are taken; one window of 128 per SM
+MANY, MANY_SHORT = 24 * WIN, 16 * WIN      # rows from which windows of 128 are taken
 
 
 @pytest.mark.parametrize("row_len", [1, 8, 9, 33])
 @pytest.mark.parametrize("rows,share", [(3, 1.0), (5, 1.0), (FEW - 1, 1.0), (FEW, 0.3), (FEW + 63, 1.0),
-                                        (FEW + 65, 0.02), (MANY - 1, 0.05), (MANY, 0.05),
-                                        (MANY + 127, 0.05), (MANY + 129, 0.0)])
+                                        (FEW + 65, 0.02), (MANY_SHORT - 1, 0.05), (MANY_SHORT + 129, 0.05),
+                                        (MANY - 1, 0.05), (MANY, 0.05), (MANY + 127, 0.05), (MANY + 129, 0.0)])
 def test_adam_rows_by_number_of_rows(rows, share, row_len):
     import torch
     abi = lib_ready()
